@@ -60,6 +60,16 @@ sem_status check_ptr(const void* p, const char* name) {
 
 namespace {
 
+int host_sm_count() {
+  static const int n = [] {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms > 0 ? sms : 1;
+  }();
+  return n;
+}
+
 // Stream-ordered allocation on `s` (the memory is usable on `s` at once and on other streams
 // once `s` has been synchronised).
 template <typename T>
@@ -114,6 +124,8 @@ void free_mesh(sem_mesh m) {
   dfree(m->coef64, h);
   dfree(m->coef32, h);
   dfree(m->G64, h);
+  dfree(m->GI, h);
+  dfree(m->gexp, h);
   dfree(m->G32, h);
   dfree(m->Gx, h);
   dfree(m->scale64, h);
@@ -156,7 +168,8 @@ std::mutex g_tune_mu;
 TuneSlot g_tune[3][SEM_MAX_N + 1];
 
 // Stored factors the local operator of precision `prec` reads: FP32 for SEM_F32; for SEM_F64X the
-// float pairs if the mesh has them, else the FP64 factors (split in the kernel); FP64 otherwise.
+// float pairs if the mesh has them, else the FP64 operator's (split in the kernel); those are FP64 values,
+// or fixed point at the orders of ax_slice_order.
 const void* stored_factors(sem_mesh m, sem_prec prec, bool* pairs) {
   *pairs = false;
   if (prec == SEM_F32) return m->G32;
@@ -164,6 +177,7 @@ const void* stored_factors(sem_mesh m, sem_prec prec, bool* pairs) {
     *pairs = true;
     return m->Gx;
   }
+  if (m->GI) return m->GI;
   return m->G64;
 }
 bool has_factors(sem_mesh m, sem_prec prec) {
@@ -198,6 +212,7 @@ sem_status launch_ax_any(sem_mesh m, sem_prec prec, sem_ax_variant v, bool cg, A
   const bool fp64_data = prec != SEM_F32;
   a.coef = fp64_data ? static_cast<const void*>(m->coef64) : static_cast<const void*>(m->coef32);
   a.G = stored_factors(m, prec, &a.g_pairs);
+  a.gexp = m->gexp;
   a.scale = fp64_data ? static_cast<const void*>(m->scale64) : static_cast<const void*>(m->scale32);
   if (v == SEM_AX_STORED && !a.G)
     return fail(SEM_ERR_ARG, "stored factors of this precision were not requested at mesh creation");
@@ -345,7 +360,15 @@ extern "C" sem_status sem_mesh_create(int N, int64_t nv, const double* vert_xyz,
     SEM_STEP(dmalloc(&bad, 1, nullptr, s));
     SEM_STEP(dmalloc(&m->coef64, static_cast<size_t>(E) * 24, &acc, s));
     SEM_STEP(dmalloc(&m->coef32, static_cast<size_t>(E) * 24, &acc, s));
-    if (flags & SEM_MESH_F64_STORED) SEM_STEP(dmalloc(&m->G64, static_cast<size_t>(E * 6 * P), &acc, s));
+    if (flags & SEM_MESH_F64_STORED) {
+      // the persistent CG kernel of small meshes (use_graph = 2) reads FP64 factors
+      if (!ax_slice_order(N) || E < host_sm_count())
+        SEM_STEP(dmalloc(&m->G64, static_cast<size_t>(E * 6 * P), &acc, s));
+      if (ax_slice_order(N)) {
+        SEM_STEP(dmalloc(&m->GI, static_cast<size_t>(E * 6 * P), &acc, s));
+        SEM_STEP(dmalloc(&m->gexp, static_cast<size_t>(E), &acc, s));
+      }
+    }
     if (flags & SEM_MESH_F64X_STORED) SEM_STEP(dmalloc(&m->Gx, static_cast<size_t>(2 * E * 6 * P), &acc, s));
     if (flags & SEM_MESH_F32_STORED)
       SEM_STEP(dmalloc(&m->G32, static_cast<size_t>(E * factor_stride(m->Np, true)), &acc, s));
@@ -394,7 +417,8 @@ extern "C" sem_status sem_mesh_create(int N, int64_t nv, const double* vert_xyz,
     SEM_CSTEP(cudaMemsetAsync(bad, 0, sizeof(int), s));
     SEM_STEP(launch_coefficients(E, Xd, m->coef64, m->coef32, s));
     // geometric factors (and the det J > 0 check at every GLL point)
-    SEM_STEP(launch_geometry(N, E, m->coef64, m->G64, m->G32, nullptr, nullptr, bad, factor_stride(m->Np, false),
+    if (m->GI) SEM_STEP(launch_fixed_factors(N, E, m->coef64, m->GI, m->gexp, bad, s));
+    if (!m->GI || m->G64 || m->G32 || m->Gx || m->scale64) SEM_STEP(launch_geometry(N, E, m->coef64, m->G64, m->G32, nullptr, nullptr, bad, factor_stride(m->Np, false),
                              factor_stride(m->Np, true), s, m->scale64, m->scale32, m->Gx));
     int bad_h = 0;
     SEM_CSTEP(cudaMemcpyAsync(&bad_h, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -820,7 +844,7 @@ sem_status cg_start(sem_cg c, const void* b, void* x, bool x0_is_zero, cudaStrea
     sem_ax_variant rv = c->variant;
     if (rp == SEM_F64X) {
       rp = SEM_F64;
-      if (rv == SEM_AX_STORED && !m->G64) rv = SEM_AX_OTF;
+      if (rv == SEM_AX_STORED && !has_factors(m, SEM_F64)) rv = SEM_AX_OTF;
     }
     SEM_TRY(launch_ax_any(m, rp, rv, false, a, s));
     SEM_TRY(launch_dssum(data_prec(c->prec), m->gs, c->w, 1, s));
@@ -875,16 +899,6 @@ sem_status cg_enqueue_iteration(sem_cg c, cudaStream_t s) {
   SEM_TRY(launch_ax_any(c->m, c->prec, c->variant, true, cg_ax_launch(c), s));
   SEM_TRY(cg_enqueue_gs(c, s));
   return cg_enqueue_update(c, s);
-}
-
-int host_sm_count() {
-  static const int n = [] {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
-  }();
-  return n;
 }
 
 // use_graph = 2: FP64 CG with stored factors on a mesh with fewer elements than the device has
@@ -1351,6 +1365,7 @@ extern "C" sem_status sem_autotune(sem_mesh m, sem_prec prec, int reps, sem_tune
         a.shape = shape == 0 ? 2 : shape;  // the tuner times each shape as it is
         a.coef = prec == SEM_F32 ? static_cast<const void*>(m->coef32) : static_cast<const void*>(m->coef64);
         a.G = stored_factors(m, prec, &a.g_pairs);
+        a.gexp = m->gexp;
         a.scale = prec == SEM_F32 ? static_cast<const void*>(m->scale32) : static_cast<const void*>(m->scale64);
         auto launch = [&] {
           if (prec == SEM_F64X) return launch_ax_f64x(m->N, v, false, a, s);

@@ -590,7 +590,10 @@ template <int NP, typename T, int EPB>
 sem_status launch_ax_shape(int N, sem_ax_variant v, bool cg, const AxLaunch& a, cudaStream_t s) {
   if (v == SEM_AX_OTF)
     return cg ? launch_ax_t<NP, T, 1, true, EPB>(N, a, s) : launch_ax_t<NP, T, 1, false, EPB>(N, a, s);
-  return cg ? launch_ax_t<NP, T, 0, true, EPB>(N, a, s) : launch_ax_t<NP, T, 0, false, EPB>(N, a, s);
+  if constexpr (std::is_same_v<T, double> && ax_slice_order(NP - 1))
+    return launch_ax_slice(N, cg, a, s);
+  else
+    return cg ? launch_ax_t<NP, T, 0, true, EPB>(N, a, s) : launch_ax_t<NP, T, 0, false, EPB>(N, a, s);
 }
 
 // Dispatch over the block shape, the variant and the mode for one order and precision

@@ -1,4 +1,4 @@
-// Double-float local operator with stored factors (FP64 values or float pairs), 2 to 7 points
+// Double-float local operator with stored factors (FP64 or fixed-point values, or float pairs), 2 to 7 points
 // per direction; the kernel is in k_ax_df.cuh, the other orders and the on-the-fly variant in
 // k_ax_df_hi.cu, k_ax_df_otf.cu and k_ax_df_otf_hi.cu (compiled in parallel).
 #include "k_ax_df.cuh"
@@ -10,7 +10,8 @@ template <int NP>
 struct DfStored {
   static sem_status run(int N, bool cg, const AxLaunch& a, cudaStream_t s) {
     if (a.g_pairs) return cg ? launch_df_t<NP, true, kGkPairs>(N, a, s) : launch_df_t<NP, false, kGkPairs>(N, a, s);
-    return cg ? launch_df_t<NP, true, kGkF64>(N, a, s) : launch_df_t<NP, false, kGkF64>(N, a, s);
+    constexpr int kGk = ax_slice_order(NP - 1) ? kGkFixed : kGkF64;
+    return cg ? launch_df_t<NP, true, kGk>(N, a, s) : launch_df_t<NP, false, kGk>(N, a, s);
   }
 };
 

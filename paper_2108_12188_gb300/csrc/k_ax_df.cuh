@@ -36,9 +36,9 @@ namespace sem {
 namespace {
 
 // Geometric factors the double-float operator takes: FP64 values (split into float pairs in the
-// kernel), float pairs stored by the mesh (SEM_MESH_F64X_STORED), or none (rebuilt on the fly
-// from the element's trilinear coefficients).
-constexpr int kGkF64 = 0, kGkPairs = 1, kGkOtf = 2;
+// kernel), float pairs stored by the mesh (SEM_MESH_F64X_STORED), none (rebuilt on the fly
+// from the element's trilinear coefficients), or 64-bit fixed point (ax_slice_order, split in the kernel).
+constexpr int kGkF64 = 0, kGkPairs = 1, kGkOtf = 2, kGkFixed = 3;
 
 // Even/odd split of D and D^T (EoMat, computed in FP64) with every entry as a float pair.
 // For the two-wide FP32 operations of sm_100 and later, the H x H blocks are also kept
@@ -301,6 +301,30 @@ struct OtfColumnDf {
   }
 };
 
+// Scales that turn fixed-point factors into float pairs: 2^(32 - sg), 2^(16 - sg), 2^-sg (0 below FP32's
+// normal range).
+struct FixedScale {
+  float s32, s16, s0;
+  __device__ __forceinline__ static float pow2f(int e) {
+    return e < -126 ? 0.f : __int_as_float((127 + min(e, 127)) << 23);
+  }
+  __device__ __forceinline__ void init(int sg) {
+    s32 = pow2f(32 - sg);
+    s16 = pow2f(16 - sg);
+    s0 = pow2f(-sg);
+  }
+  // X = (hi & ~7) 2^32 + ((hi & 7) 2^16 + lo >> 16) 2^16 + (lo & 0xffff), three exact floats (|hi| <= 2^27),
+  // added into a pair: 48 bits of the value itself
+  __device__ __forceinline__ df2 pair(int2 x, float f) const {
+    const float a = static_cast<float>(x.y & ~7) * s32;
+    const float b = static_cast<float>(((x.y & 7) << 16) + (x.x >> 16)) * s16;
+    const float c = static_cast<float>(x.x & 0xffff) * s0;
+    const float h = __fadd_rn(a, b);
+    const float l = __fadd_rn(__fadd_rn(__fsub_rn(a, h), b), c);
+    return {h * f, l * f};
+  }
+};
+
 // Factor values staged in shared memory per element: the first three arrays (G11, G12, G13)
 // when P is even (their bytes are then a multiple of 16, as bulk copies need), all six
 // otherwise. Unstaged arrays are prefetched into L2 with the copy and read from there. The
@@ -346,7 +370,8 @@ template <int NP, bool CG, int GK>
 __global__ void __launch_bounds__(NP * NP * ax_epb<NP>(),
                                   (NP == 8 && (CG || GK != kGkOtf)) ? 4 : GK == kGkOtf ? 0 : 1)
     k_ax_df(const __grid_constant__ DfTab<NP> tab, int64_t E, const double* __restrict__ u, double* __restrict__ w,
-            const double* __restrict__ G, const double* __restrict__ coef, const double* __restrict__ r,
+            const double* __restrict__ G, const int* __restrict__ gexp, const double* __restrict__ coef,
+            const double* __restrict__ r,
             double* __restrict__ p,
             const double* __restrict__ minv, double* __restrict__ x, CgScalars* __restrict__ st,
             double* __restrict__ partials, int* __restrict__ err) {
@@ -481,6 +506,13 @@ __global__ void __launch_bounds__(NP * NP * ax_epb<NP>(),
       const double* gE = sG + slot * GST;
       const double* gH = G + (valid ? e : int64_t(0)) * 6 * P;  // arrays 3..5 from L2 when not staged
       df2 rR[NP], rS[NP];
+      FixedScale fx;
+      float fi = 1.f, fj = 1.f;
+      if constexpr (GK == kGkFixed) {
+        fx.init(valid ? __ldg(gexp + e) : 0);
+        fi = FixedScale::pow2f(-fixed_row_scale(NP, i));
+        fj = FixedScale::pow2f(-fixed_row_scale(NP, j));
+      }
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
         const int at = Stage<NP>::at(i, j, k);
@@ -490,12 +522,16 @@ __global__ void __launch_bounds__(NP * NP * ax_epb<NP>(),
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
         df2 g[6];
+        const float fk = GK == kGkFixed ? FixedScale::pow2f(-fixed_row_scale(NP, k)) : 1.f;
 #pragma unroll
         for (int m = 0; m < 6; ++m) {
           const double* src = (GST != 6 * P && m >= 3) ? gH : gE;
           if constexpr (GK == kGkPairs) {  // factors stored as float pairs: no split needed
             const float2 v = reinterpret_cast<const float2*>(src)[m * P + k * NP2 + tid];
             g[m] = {v.x, v.y};
+          } else if constexpr (GK == kGkFixed) {
+            const float fa = m < 3 ? fi : m < 5 ? fj : fk, fb = m == 0 ? fi : m == 1 || m == 3 ? fj : fk;
+            g[m] = fx.pair(reinterpret_cast<const int2*>(src)[m * P + k * NP2 + tid], fa * fb);
           } else {
             g[m] = df_from_double(src[m * P + k * NP2 + tid]);
           }
@@ -595,7 +631,7 @@ sem_status launch_df_t(int N, const AxLaunch& a, cudaStream_t s) {
   if (a.grid_out) *a.grid_out = grid;
   k_ax_df<NP, CG, GK><<<grid, NP * NP * EPB, smem, s>>>(
       make_df_tab<NP>(N), a.E, static_cast<const double*>(a.u), static_cast<double*>(a.w),
-      static_cast<const double*>(a.G), static_cast<const double*>(a.coef), static_cast<const double*>(a.r),
+      static_cast<const double*>(a.G), a.gexp, static_cast<const double*>(a.coef), static_cast<const double*>(a.r),
       static_cast<double*>(a.p), static_cast<const double*>(a.minv), static_cast<double*>(a.x), a.st, a.partials,
       a.err);
   count_launch();

@@ -9,7 +9,8 @@ template <int NP>
 struct DfStored {
   static sem_status run(int N, bool cg, const AxLaunch& a, cudaStream_t s) {
     if (a.g_pairs) return cg ? launch_df_t<NP, true, kGkPairs>(N, a, s) : launch_df_t<NP, false, kGkPairs>(N, a, s);
-    return cg ? launch_df_t<NP, true, kGkF64>(N, a, s) : launch_df_t<NP, false, kGkF64>(N, a, s);
+    constexpr int kGk = ax_slice_order(NP - 1) ? kGkFixed : kGkF64;
+    return cg ? launch_df_t<NP, true, kGk>(N, a, s) : launch_df_t<NP, false, kGk>(N, a, s);
   }
 };
 

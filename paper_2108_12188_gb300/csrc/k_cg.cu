@@ -223,20 +223,23 @@ __global__ void k_cg_update(int64_t n, T* __restrict__ x, const T* __restrict__ 
   if constexpr (sizeof(T) == 8) {
     // x, r, z: three FP64 operations per point. <r, z, c> and <r, r, c>: r and z as float
     // pairs (integer split), c as a float pair from a shared table, (c r) an error-free
-    // product, then rz += (c r) z and rr += (c r) r in double-float.
+    // product, then rz += (c r) z and rr += (c r) r in double-float. The splits are rounded and every
+    // product term is kept: cut off, they shift both sums by about 1e-14 the same way at every
+    // point, and with them alpha and beta (x after 10 iterations on 8^3 elements: 5.1e-14 off a long-double
+    // computation with the cut-off, 3.9e-15 without, in the same time).
     __shared__ df2 sC[256];
-    for (int m = threadIdx.x; m < 256; m += blockDim.x) sC[m] = m == 1 ? df2{1.f, 0.f} : df_from_double(ctab[m]);
+    for (int m = threadIdx.x; m < 256; m += blockDim.x) sC[m] = m == 1 ? df2{1.f, 0.f} : df_split<true>(ctab[m]);
     __syncthreads();
     df2 rz{0.f, 0.f}, rr{0.f, 0.f};
     sweep([&](T& xi, T pi, T& ri, T wi, T& zi, T mi, unsigned m) {
       if constexpr (!FUSED) xi += alpha * pi;
       ri = ri - alpha * wi;
       zi = minv ? mi * ri : ri;
-      const df2 r2 = df_from_double(ri), z2 = df_from_double(zi), c2 = sC[m];
+      const df2 r2 = df_split<true>(ri), z2 = df_split<true>(zi), c2 = sC[m];
       float ch, cl;
       df_prod(c2.h, c2.l, r2.h, r2.l, ch, cl);
-      df_fma_acc(rz, ch, cl, z2.h, z2.l);
-      df_fma_acc(rr, ch, cl, r2.h, r2.l);
+      df_fma_acc_full(rz, ch, cl, z2.h, z2.l);
+      df_fma_acc_full(rr, ch, cl, r2.h, r2.l);
     });
     v[0] = block_sum(static_cast<double>(rz.h) + static_cast<double>(rz.l), sRed);
     v[1] = block_sum(static_cast<double>(rr.h) + static_cast<double>(rr.l), sRed);

@@ -126,6 +126,42 @@ __global__ void k_geometry(const __grid_constant__ GllAll tab, int Np, int64_t E
   if (S32) S32[idx] = static_cast<float>(sc);
 }
 
+// G of one element per block as the fixed point of ax_slice_order: sg = 59 - (exponent of the
+// element's largest entry, row scales included). sG: 6 P doubles of dynamic shared memory.
+__global__ void k_fixed_factors(const __grid_constant__ GllAll tab, int Np, const double* __restrict__ coef,
+                                int2* __restrict__ X, int* __restrict__ gexp, int* __restrict__ bad) {
+  extern __shared__ double sG[];
+  __shared__ int sTop;
+  const int P = Np * Np * Np;
+  const int64_t e = blockIdx.x;
+  if (threadIdx.x == 0) sTop = -4000;
+  __syncthreads();
+  int top = -4000;
+  for (int r = threadIdx.x; r < P; r += blockDim.x) {
+    const int i = r % Np, j = (r / Np) % Np, k = r / (Np * Np);
+    double G[6], B, det;
+    point_geometry(coef + e * 24, tab.xi[i], tab.xi[j], tab.xi[k], tab.w[i] * tab.w[j] * tab.w[k], G, &B, &det);
+    if (!(det > 0.0) || !isfinite(det)) atomicOr(bad, 1);
+    const int c[3] = {fixed_row_scale(Np, i), fixed_row_scale(Np, j), fixed_row_scale(Np, k)};
+    for (int m = 0; m < 6; ++m) {
+      const double g = scalbn(G[m], c[m < 3 ? 0 : m < 5 ? 1 : 2] + c[m < 3 ? m : m < 5 ? m - 2 : 2]);
+      sG[m * P + r] = g;
+      int ex = -4000;
+      if (g != 0.0 && isfinite(g)) frexp(g, &ex);
+      top = max(top, ex);
+    }
+  }
+  atomicMax(&sTop, top);
+  __syncthreads();
+  const int sg = 59 - sTop;
+  for (int q = threadIdx.x; q < 6 * P; q += blockDim.x) {
+    const long long x = __double2ll_rn(scalbn(sG[q], sg));
+    const int lo = static_cast<int>(static_cast<uint32_t>(x));
+    X[e * 6 * P + q] = make_int2(lo, static_cast<int>((x - lo) >> 32));
+  }
+  if (threadIdx.x == 0) gexp[e] = sg;
+}
+
 __global__ void k_coords(const __grid_constant__ GllAll tab, int Np, int64_t E, const double* __restrict__ coef,
                          double* __restrict__ xyz, int64_t n) {
   const int64_t P = static_cast<int64_t>(Np) * Np * Np;
@@ -243,6 +279,15 @@ sem_status launch_geometry(int N, int64_t E, const double* coef64, double* G64, 
   const int64_t n = E * Np * Np * Np;
   k_geometry<<<ceil_div(n, kThreads), kThreads, 0, s>>>(gll_all(N), Np, E, coef64, G64, G32, B64, B32, bad, gs64,
                                                         gs32, S64, S32, GX);
+  count_launch();
+  SEM_CUDA_TRY(cudaGetLastError());
+  return SEM_OK;
+}
+
+sem_status launch_fixed_factors(int N, int64_t E, const double* coef64, int2* X, int* gexp, int* bad, cudaStream_t s) {
+  const int P = (N + 1) * (N + 1) * (N + 1);  // 24 KB of shared memory at N = 7, the largest ax_slice_order
+  k_fixed_factors<<<static_cast<unsigned>(E), P < 128 ? 64 : 128, 6 * static_cast<size_t>(P) * sizeof(double), s>>>(
+      gll_all(N), N + 1, coef64, X, gexp, bad);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;

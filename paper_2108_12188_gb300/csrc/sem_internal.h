@@ -133,6 +133,19 @@ inline int64_t factor_stride(int Np, bool fp32) {
   return fp32 ? (s + 3) / 4 * 4 : s;
 }
 
+// Orders whose FP64 stored-factor operator runs on the tensor cores (k_ax_slice.cuh). Their meshes
+// keep G as 64-bit fixed point instead of FP64, in the same bytes: X = G_ab 2^(sg + c_a + c_b), |X| <=
+// 2^59, as 32-bit signed halves (low, high), with sg per element and c = fixed_row_scale of the
+// point's index along each direction. At 16.8M points the FP64 kernel against this one: N = 3 1.12 and
+// 0.36 ms, N = 5 1.50 and 0.79, N = 6 1.52 and 0.62, N = 7 1.50 and 0.36. N = 2 and 4 fill too little of
+// the 8 x 8 x 8 points a block works on (0.86 against 0.93 ms, 1.13 against 1.31). At N = 1 the FP64
+// differences of equal values are exact zeros, which fixed-point factors do not keep on stretched
+// elements (relative error 1.4e-15 against 1.2e-16 at aspect ratio 100).
+constexpr bool ax_slice_order(int N) { return N == 3 || N == 5 || N == 6 || N == 7; }
+__host__ __device__ constexpr int fixed_row_scale(int NP, int i) {
+  return i == 0 || i == NP - 1 ? (NP <= 4 ? 1 : 2) : 0;
+}
+
 // ---- reduction scratch ----
 constexpr int kRedMax = 8192;  // upper bound of blocks of any reducing launch
 
@@ -222,7 +235,9 @@ struct sem_mesh_s {
   // device arrays
   double* coef64 = nullptr;   // [E][24] trilinear coefficients a0..a7 (x, y, z)
   float* coef32 = nullptr;    // [E][24] rounded to FP32
-  double* G64 = nullptr;      // [E][6][P] or null
+  double* G64 = nullptr;      // [E][6][P] or null (ax_slice_order: only for fewer elements than SMs)
+  int2* GI = nullptr;         // [E][6][P] fixed-point factors (ax_slice_order) or null
+  int* gexp = nullptr;        // [E] their exponents sg
   float* G32 = nullptr;       // [E][factor_stride] (the [6][P] block, padded to 16 bytes) or null
   float* Gx = nullptr;        // [E][6][P] float pairs (high, low) of G for SEM_F64X, or null
   double* scale64 = nullptr;  // [n] w_i w_j w_k / det J (SEM_MESH_OTF_SCALE) or null
@@ -272,7 +287,8 @@ struct AxLaunch {
   const void* u;      // input (plain mode)
   void* w;            // output
   const void* G;      // stored factors or null
-  bool g_pairs;       // SEM_F64X: G holds float pairs (high, low) instead of FP64 values
+  bool g_pairs;       // SEM_F64X: G holds float pairs (high, low) instead of the FP64 operator's factors
+  const int* gexp;    // exponents of fixed-point factors (ax_slice_order)
   const void* coef;   // trilinear coefficients (otf)
   const void* scale;  // per-point w/det J (otf with stored scale)
   // CG mode (p = z + beta p prologue, <p, w> partials in the epilogue)
@@ -294,7 +310,10 @@ sem_status launch_ax_f64_lo(int N, sem_ax_variant v, bool cg_mode, const AxLaunc
 sem_status launch_ax_f64_hi(int N, sem_ax_variant v, bool cg_mode, const AxLaunch& a, cudaStream_t s);  // N+1 >= 8
 sem_status launch_ax_f32_lo(int N, sem_ax_variant v, bool cg_mode, const AxLaunch& a, cudaStream_t s);
 sem_status launch_ax_f32_hi(int N, sem_ax_variant v, bool cg_mode, const AxLaunch& a, cudaStream_t s);
+// FP64 with stored (fixed-point) factors on the tensor cores, ax_slice_order only.
+sem_status launch_ax_slice(int N, bool cg_mode, const AxLaunch& a, cudaStream_t s);
 inline sem_status launch_ax_f64(int N, sem_ax_variant v, bool cg, const AxLaunch& a, cudaStream_t s) {
+  if (v == SEM_AX_STORED && ax_slice_order(N)) return launch_ax_slice(N, cg, a, s);
   return N + 1 <= 7 ? launch_ax_f64_lo(N, v, cg, a, s) : launch_ax_f64_hi(N, v, cg, a, s);
 }
 inline sem_status launch_ax_f32(int N, sem_ax_variant v, bool cg, const AxLaunch& a, cudaStream_t s) {
@@ -349,6 +368,8 @@ sem_status launch_coefficients(int64_t E, const double* X, double* coef64, float
 sem_status launch_geometry(int N, int64_t E, const double* coef64, double* G64, float* G32, double* B64,
                            float* B32, int* bad_flag, int64_t gs64, int64_t gs32, cudaStream_t s,
                            double* S64 = nullptr, float* S32 = nullptr, float* GX = nullptr);
+// Fixed-point factors and their exponents (ax_slice_order), with the det J > 0 check.
+sem_status launch_fixed_factors(int N, int64_t E, const double* coef64, int2* X, int* gexp, int* bad_flag, cudaStream_t s);
 sem_status launch_coords(int N, int64_t E, const double* coef64, double* xyz, int64_t n, cudaStream_t s);
 sem_status launch_local_diag(int N, int64_t E, const double* coef64, double* d, cudaStream_t s);
 sem_status launch_rhs_local(int N, int64_t E, const double* coef64, int a, int b, int c, double* out,
