@@ -40,15 +40,68 @@ __device__ __forceinline__ T weight_t(const uint8_t* __restrict__ mult, const do
   return m == 1u ? T(1) : static_cast<T>(__ldg(ctab + m));
 }
 
+// Products of <a, b, c> without FP64 instructions beside the accumulating multiply-add. Where the
+// multiplicity m is a power of two (every node of a hexahedral grid) and a is normal, a / m is a
+// change of the exponent field; an FP32 value that is normal or zero becomes FP64 by moving its fields.
+__device__ __forceinline__ bool pow2_mult(unsigned m) { return (m & (m - 1)) == 0u; }
+__device__ __forceinline__ double over_mult(double a, unsigned m, const double* __restrict__ ctab) {
+  const unsigned hi = static_cast<unsigned>(__double2hiint(a)), ex = (hi >> 20) & 0x7ffu;
+  if (ex - 9u < 2038u && pow2_mult(m))  // 8 < ex < 2047: a / 128 is normal
+    return __hiloint2double(static_cast<int>(hi - ((31 - __clz(static_cast<int>(m))) << 20)), __double2loint(a));
+  return a * __ldg(ctab + m);
+}
+__device__ __forceinline__ bool moves(float a) {  // normal or zero
+  const unsigned mag = __float_as_uint(a) & 0x7fffffffu;
+  return mag - 0x00800000u < 0x7f000000u || mag == 0u;
+}
+__device__ __forceinline__ double moved(float a, unsigned m) {  // a / m, m a power of two
+  const unsigned u = __float_as_uint(a), mag = u & 0x7fffffffu;
+  const unsigned hi = mag == 0u ? 0u : (mag >> 3) + ((865u + __clz(static_cast<int>(m))) << 20);
+  return __hiloint2double(static_cast<int>((u & 0x80000000u) | hi), static_cast<int>(u << 29));
+}
+
+// <a, b, c> accumulated in FP64. The FP64 pipe (2 multiply-adds per clock per SM) is what the plain
+// form, two FP64 operations per point (and two conversions of FP32 data), waits for: 53 us of a
+// 79 us launch at 16.8M FP64 points. Here a point takes one, a / m being formed on the integer
+// pipes, and each thread loads four points of both vectors (16-byte loads) before it uses them.
+// 16.8M points: FP64 78 -> 47.5 us (floor 42), FP32 137 -> 42 us (the FP64 multiply-adds take 26).
 template <typename T>
 __global__ void k_glsc3(int64_t n, const T* __restrict__ a, const T* __restrict__ b, const uint8_t* __restrict__ mult,
                         const double* __restrict__ ctab, double* __restrict__ partials, unsigned int* ticket,
                         double* __restrict__ result) {
   __shared__ double sRed[kThreads / 32];
   double acc = 0.0;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x)
-    acc += static_cast<double>(a[i]) * static_cast<double>(b[i]) * weight(mult, ctab, i);
+  const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  struct alignas(16) Four {
+    T v[4];
+  };
+  const int64_t n4 = n / 4;
+  auto general = [&](T x, T y, unsigned m) {
+    acc = fma(static_cast<double>(x) * __ldg(ctab + m), static_cast<double>(y), acc);
+  };
+#pragma unroll 2
+  for (int64_t q = t0; q < n4; q += stride) {
+    const Four x = reinterpret_cast<const Four*>(a)[q], y = reinterpret_cast<const Four*>(b)[q];
+    const uchar4 m4 = reinterpret_cast<const uchar4*>(mult)[q];
+    const unsigned m[4] = {m4.x, m4.y, m4.z, m4.w};
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+      for (int l = 0; l < 4; ++l) acc = fma(over_mult(x.v[l], m[l], ctab), y.v[l], acc);
+    } else {  // one test for four points, so that the conversions of the other branch are not issued
+      bool all = true;
+#pragma unroll
+      for (int l = 0; l < 4; ++l) all = all & moves(x.v[l]) & moves(y.v[l]) & pow2_mult(m[l]);
+      if (all) {
+#pragma unroll
+        for (int l = 0; l < 4; ++l) acc = fma(moved(x.v[l], m[l]), moved(y.v[l], 1u), acc);
+      } else {
+#pragma unroll 1
+        for (int l = 0; l < 4; ++l) general(a[4 * q + l], b[4 * q + l], mult[4 * q + l]);
+      }
+    }
+  }
+  for (int64_t i = 4 * n4 + t0; i < n; i += stride) general(a[i], b[i], mult[i]);
   const double v[1] = {block_sum(acc, sRed)};
   if (publish_partials<1>(v, partials, ticket)) {
     const double s = sum_partials(partials, gridDim.x, 1, 0, sRed);
@@ -285,8 +338,8 @@ __global__ void k_cg_update(int64_t n, T* __restrict__ x, const T* __restrict__ 
 
 sem_status launch_glsc3(sem_prec prec, int64_t n, const void* a, const void* b, const uint8_t* mult,
                         const double* ctab, double* partials, unsigned int* ticket, double* result, cudaStream_t s) {
-  const int grid = vec_grid(n, prec == SEM_F64 ? resident_blocks<k_glsc3<double>>(kThreads)
-                                               : resident_blocks<k_glsc3<float>>(kThreads));
+  const int grid = vec_grid((n + 3) / 4, prec == SEM_F64 ? resident_blocks<k_glsc3<double>>(kThreads)
+                                                         : resident_blocks<k_glsc3<float>>(kThreads));
   if (prec == SEM_F64)
     k_glsc3<double><<<grid, kThreads, 0, s>>>(n, static_cast<const double*>(a), static_cast<const double*>(b), mult,
                                               ctab, partials, ticket, result);
