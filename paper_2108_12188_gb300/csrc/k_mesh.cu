@@ -207,26 +207,130 @@ __global__ void k_local_diag(const __grid_constant__ GllTable tab, int Np, int64
   }
 }
 
-// (B f)(x) with f = (a^2+b^2+c^2) pi^2 sin(a pi x) sin(b pi y) sin(c pi z).
-__global__ void k_rhs_local(const __grid_constant__ GllAll tab, int Np, int64_t E, const double* __restrict__ coef,
-                            int fa, int fb, int fc, double* __restrict__ out) {
-  const int64_t P = static_cast<int64_t>(Np) * Np * Np;
-  const int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (idx >= E * P) return;
-  const int64_t e = idx / P;
-  const int r = static_cast<int>(idx - e * P);
-  const int i = r % Np, j = (r / Np) % Np, k = r / (Np * Np);
-  const double xi = tab.xi[i], eta = tab.xi[j], gam = tab.xi[k];
-  const double* a = coef + e * 24;
-  double x[3];
-  for (int c = 0; c < 3; ++c)
-    x[c] = a[c] + a[3 + c] * xi + a[6 + c] * eta + a[9 + c] * gam + a[12 + c] * xi * eta + a[15 + c] * xi * gam +
-           a[18 + c] * eta * gam + a[21 + c] * xi * eta * gam;
-  double G[6], B, det;
-  point_geometry(a, xi, eta, gam, tab.w[i] * tab.w[j] * tab.w[k], G, &B, &det);
-  const double pi2 = 9.869604401089358;  // pi^2
-  const double f = (fa * fa + fb * fb + fc * fc) * pi2 * sinpi(fa * x[0]) * sinpi(fb * x[1]) * sinpi(fc * x[2]);
-  out[idx] = B * f;
+// (-1)^(n / 2) / n!, the coefficients of the sine's and cosine's Taylor sums.
+struct TaylorTab {
+  double v[18];
+};
+TaylorTab taylor_tab() {
+  TaylorTab t{};
+  double f = 1.0;
+  for (int n = 0; n < 18; ++n) {
+    if (n > 0) f /= n;
+    t.v[n] = n / 2 % 2 ? -f : f;
+  }
+  return t;
+}
+
+// Terms of the sums that leave less than 2^-55 out for |t| <= pi slope; 0: too large for them.
+__device__ __forceinline__ int taylor_terms(double slope) {
+  const double a = fabs(slope);
+  return a <= 1.0 / 32 ? 4 : a <= 1.0 / 16 ? 5 : a <= 1.0 / 8 ? 6 : a <= 1.0 / 4 ? 8 : 0;
+}
+// sin t and cos t up to t^(2 terms + 1) and t^(2 terms).
+__device__ __forceinline__ void sincos_small(const TaylorTab& k, int terms, double t, double* s, double* c) {
+  const double t2 = t * t;
+  double p = k.v[2 * terms + 1], q = k.v[2 * terms];
+#pragma unroll 1
+  for (int n = terms - 1; n >= 1; --n) {
+    p = fma(p, t2, k.v[2 * n + 1]);
+    q = fma(q, t2, k.v[2 * n]);
+  }
+  *s = fma(t * t2, p, t);
+  *c = fma(t2, q, 1.0);
+}
+
+// (B f)(x) with f = (a^2+b^2+c^2) pi^2 sin(a pi x) sin(b pi y) sin(c pi z), `split` threads per i-row of an
+// element (each every split-th pair of points +-xi), epb elements per block or, for chunk < rows, `chunk`
+// rows of one element. The kernel is bound by
+// FP64 instructions (2 multiply-adds per clock per SM), and three sinpi and the Jacobian at every point
+// are 190 of them. Along a row x is linear in xi, so sin(a pi x) is a rotation of the row's midpoint value
+// by angles +-a pi B xi_i, whose sines and cosines are short sums and serve two points each (the GLL nodes
+// are symmetric); the midpoints follow the same way from one value per k-plane. Along the row det J is a
+// quadratic in xi, formed once. 48 instructions per point at N = 9: with the gather-scatter 2.14 ->
+// 0.85 ms at 8.0M points (0.72 of it at the FP64 rate a chain of multiply-adds reaches). Elements too large for the short sums (|a B| > 1/4) take sincospi and sinpi.
+__global__ void k_rhs_local(const __grid_constant__ GllAll tab, const __grid_constant__ TaylorTab tay, int Np, int epb,
+                            int split, int chunk, int64_t E, const double* __restrict__ coef, int fa, int fb, int fc,
+                            double* __restrict__ out) {
+  extern __shared__ double sh[];  // [epb][P] values, then [epb][Np][3] (sin, cos) of the planes' midpoints
+  constexpr double kPi = 3.14159265358979323846;
+  const int P = Np * Np * Np, rows = Np * Np;
+  double2* plane = reinterpret_cast<double2*>(sh + static_cast<size_t>(epb) * P + (static_cast<size_t>(epb) * P) % 2);
+  const int parts = (rows + chunk - 1) / chunk, row0 = blockIdx.x % parts * chunk;  // (parts > 1: epb = 1)
+  const int64_t e0 = static_cast<int64_t>(blockIdx.x / parts) * epb;
+  const int count = static_cast<int>(E - e0 < epb ? E - e0 : epb);
+  const int my_rows = parts > 1 ? min(chunk, rows - row0) : count * rows;
+  const double f[3] = {static_cast<double>(fa), static_cast<double>(fb), static_cast<double>(fc)};
+  for (int q = threadIdx.x; q < count * Np * 3; q += blockDim.x) {
+    const int c = q % 3, k = q / 3 % Np;
+    const double* a = coef + (e0 + q / (3 * Np)) * 24;
+    double s, co;
+    sincospi(f[c] * fma(a[9 + c], tab.xi[k], a[c]), &s, &co);
+    plane[q] = make_double2(s, co);
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < my_rows * split; q += blockDim.x) {
+    const int part = q % split, row = row0 + q / split, el = row / rows, j = row % rows % Np, k = row % rows / Np;
+    const double* a = coef + (e0 + el) * 24;
+    const double eta = tab.xi[j], gam = tab.xi[k], eg = eta * gam;
+    double g0[3], p[3], pq[3], r[3], rs[3], S[3], C[3], base[3], turn[3];
+    int terms[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double a1 = a[3 + c], a2 = a[6 + c], a3 = a[9 + c], a4 = a[12 + c], a5 = a[15 + c], a6 = a[18 + c],
+                   a7 = a[21 + c];
+      g0[c] = a1 + a4 * eta + a5 * gam + a7 * eg;  // dx/dxi, constant along the row
+      p[c] = a2 + a6 * gam;                        // dx/deta = p + xi pq
+      pq[c] = a4 + a7 * gam;
+      r[c] = a3 + a6 * eta;                        // dx/dgam = r + xi rs
+      rs[c] = a5 + a7 * eta;
+      const double mid = fma(a3, gam, a[c]), up = f[c] * p[c];
+      const double2 m = plane[(el * Np + k) * 3 + c];
+      S[c] = m.x;
+      C[c] = m.y;
+      base[c] = f[c] * fma(p[c], eta, mid);
+      if (const int n = taylor_terms(up)) {
+        double ds, dc;
+        sincos_small(tay, n, kPi * up * eta, &ds, &dc);
+        S[c] = fma(m.x, dc, m.y * ds);
+        C[c] = fma(m.y, dc, -m.x * ds);
+      } else {
+        sincospi(base[c], &S[c], &C[c]);
+      }
+      const double along = f[c] * g0[c];
+      terms[c] = taylor_terms(along);
+      turn[c] = terms[c] ? kPi * along : along;
+    }
+    double h1[3], h2[3];  // det J = (p + xi pq) . ((r + xi rs) cross g0)
+    cross3(r, g0, h1);
+    cross3(rs, g0, h2);
+    auto dot = [](const double* x, const double* y) { return x[0] * y[0] + x[1] * y[1] + x[2] * y[2]; };
+    const double pi2 = 9.869604401089358;  // pi^2
+    const double w = tab.w[j] * tab.w[k] * ((fa * fa + fb * fb + fc * fc) * pi2);
+    const double d0 = w * dot(p, h1), d1 = w * (dot(p, h2) + dot(pq, h1)), d2 = w * dot(pq, h2);
+    double* o = sh + (row - row0) * Np;
+#pragma unroll 1
+    for (int i = part; 2 * i < Np; i += split) {
+      const double xi = tab.xi[i];
+      double lo = tab.w[i], hi = lo;  // the points xi and -xi
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if (terms[c]) {
+          double ds, dc;
+          sincos_small(tay, terms[c], turn[c] * xi, &ds, &dc);
+          const double sc = S[c] * dc;
+          lo *= fma(C[c], ds, sc);
+          hi *= fma(-C[c], ds, sc);
+        } else {
+          lo *= sinpi(fma(turn[c], xi, base[c]));
+          hi *= sinpi(fma(turn[c], -xi, base[c]));
+        }
+      }
+      o[i] = lo * fma(xi, fma(xi, d2, d1), d0);
+      o[Np - 1 - i] = hi * fma(-xi, fma(-xi, d2, d1), d0);
+    }
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < my_rows * Np; q += blockDim.x) out[e0 * P + row0 * Np + q] = sh[q];
 }
 
 template <typename T>
@@ -251,14 +355,19 @@ __global__ void k_cast(int64_t n, const double* __restrict__ in, float* __restri
     out[i] = static_cast<float>(in[i]);
 }
 
-// One thread per item, at most 32 blocks per SM (grid-stride beyond).
-int grid_for(int64_t n) {
-  static const int cap = [] {
+int sm_count() {
+  static const int n = [] {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return 32 * (sms > 0 ? sms : 1);
+    return sms > 0 ? sms : 1;
   }();
+  return n;
+}
+
+// One thread per item, at most 32 blocks per SM (grid-stride beyond).
+int grid_for(int64_t n) {
+  const int cap = 32 * sm_count();
   const int64_t b = (n + kThreads - 1) / kThreads;
   return static_cast<int>(b < cap ? (b > 0 ? b : 1) : cap);
 }
@@ -314,9 +423,24 @@ sem_status launch_local_diag(int N, int64_t E, const double* coef64, double* d, 
 }
 
 sem_status launch_rhs_local(int N, int64_t E, const double* coef64, int a, int b, int c, double* out, cudaStream_t s) {
-  const int Np = N + 1;
-  const int64_t n = E * Np * Np * Np;
-  k_rhs_local<<<ceil_div(n, kThreads), kThreads, 0, s>>>(gll_all(N), Np, E, coef64, a, b, c, out);
+  constexpr int kBlock = 128;
+  const int Np = N + 1, P = Np * Np * Np, rows = Np * Np;
+  // Meshes whose rows do not give every scheduler four warps: a thread per pair of points (the row's share
+  // of the work repeated) and blocks of one pass over at most 128 of them, for a short chain on many
+  // SMs (4^3 elements at N = 7, with the gather-scatter: 21 us; a thread per row 35 us).
+  const int split = E * rows < static_cast<int64_t>(sm_count()) * 512 ? (Np + 1) / 2 : 1;
+  const int chunk = split > 1 ? kBlock / split : rows;
+  // elements per block: the fewest idle lanes in the block's last pass over its rows, 32 KB of values at most
+  int epb = 1;
+  auto waste = [&](int q) { return 1.0 - static_cast<double>(q) * rows / (ceil_div(static_cast<int64_t>(q) * rows, kBlock) * kBlock); };
+  if (split == 1)
+    for (int q = 2; q * P <= 4096; ++q)
+      if (waste(q) < waste(epb) - 1e-9) epb = q;
+  const size_t smem = (static_cast<size_t>(epb) * P + 1 + 6 * static_cast<size_t>(epb) * Np) * sizeof(double);
+  static const TaylorTab tay = taylor_tab();
+  const int64_t blocks = split > 1 ? E * ceil_div(rows, chunk) : ceil_div(E, epb);
+  k_rhs_local<<<static_cast<unsigned>(blocks), kBlock, smem, s>>>(gll_all(N), tay, Np, epb, split,
+                                                                  chunk < rows ? chunk : rows, E, coef64, a, b, c, out);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;
