@@ -169,10 +169,11 @@ TuneSlot g_tune[3][SEM_MAX_N + 1];
 
 // Stored factors the local operator of precision `prec` reads: FP32 for SEM_F32; for SEM_F64X the
 // float pairs if the mesh has them, else the FP64 operator's (split in the kernel); those are FP64 values,
-// or fixed point at the orders of ax_slice_order.
+// or fixed point at the orders of ax_slice_order (one array for both precisions where f64x_on_slices).
 const void* stored_factors(sem_mesh m, sem_prec prec, bool* pairs) {
   *pairs = false;
   if (prec == SEM_F32) return m->G32;
+  if (prec == SEM_F64 && !(m->flags & SEM_MESH_F64_STORED)) return nullptr;
   if (prec == SEM_F64X && m->Gx) {
     *pairs = true;
     return m->Gx;
@@ -360,16 +361,16 @@ extern "C" sem_status sem_mesh_create(int N, int64_t nv, const double* vert_xyz,
     SEM_STEP(dmalloc(&bad, 1, nullptr, s));
     SEM_STEP(dmalloc(&m->coef64, static_cast<size_t>(E) * 24, &acc, s));
     SEM_STEP(dmalloc(&m->coef32, static_cast<size_t>(E) * 24, &acc, s));
-    if (flags & SEM_MESH_F64_STORED) {
-      // the persistent CG kernel of small meshes (use_graph = 2) reads FP64 factors
-      if (!ax_slice_order(N) || E < host_sm_count())
-        SEM_STEP(dmalloc(&m->G64, static_cast<size_t>(E * 6 * P), &acc, s));
-      if (ax_slice_order(N)) {
-        SEM_STEP(dmalloc(&m->GI, static_cast<size_t>(E * 6 * P), &acc, s));
-        SEM_STEP(dmalloc(&m->gexp, static_cast<size_t>(E), &acc, s));
-      }
+    // (the persistent CG kernel of small meshes, use_graph = 2, reads FP64 factors at every order)
+    if ((flags & SEM_MESH_F64_STORED) && (!ax_slice_order(N) || E < host_sm_count()))
+      SEM_STEP(dmalloc(&m->G64, static_cast<size_t>(E * 6 * P), &acc, s));
+    const bool x_fixed = (flags & SEM_MESH_F64X_STORED) && f64x_on_slices(N);
+    if (((flags & SEM_MESH_F64_STORED) && ax_slice_order(N)) || x_fixed) {
+      SEM_STEP(dmalloc(&m->GI, static_cast<size_t>(E * 6 * P), &acc, s));
+      SEM_STEP(dmalloc(&m->gexp, static_cast<size_t>(E), &acc, s));
     }
-    if (flags & SEM_MESH_F64X_STORED) SEM_STEP(dmalloc(&m->Gx, static_cast<size_t>(2 * E * 6 * P), &acc, s));
+    if ((flags & SEM_MESH_F64X_STORED) && !x_fixed)
+      SEM_STEP(dmalloc(&m->Gx, static_cast<size_t>(2 * E * 6 * P), &acc, s));
     if (flags & SEM_MESH_F32_STORED)
       SEM_STEP(dmalloc(&m->G32, static_cast<size_t>(E * factor_stride(m->Np, true)), &acc, s));
     if (flags & SEM_MESH_OTF_SCALE) {
@@ -722,6 +723,8 @@ struct sem_cg_s {
 namespace sem {
 namespace {
 
+bool cg_fused(sem_cg c) { return fused_cg(c->prec, c->m->N, c->variant); }
+
 const void* minv_of(sem_cg c) {
   if (!c->precond) return nullptr;
   return c->prec == SEM_F32 ? static_cast<const void*>(c->m->minv32) : static_cast<const void*>(c->m->minv64);
@@ -756,6 +759,8 @@ void cg_free(sem_cg c) {
 sem_status cg_alloc(sem_mesh m, sem_prec prec, sem_ax_variant v, int precond, double rtol, int max_iter, int use_graph,
                     sem_cg* out) {
   *out = nullptr;
+  int shape;
+  resolve_variant(m, prec, v, &v, &shape);  // SEM_AX_AUTO: one variant for the handle's life
   if (v == SEM_AX_STORED && !has_factors(m, prec))
     return fail(SEM_ERR_ARG, "stored factors of this precision were not requested at mesh creation");
   if (prec == SEM_F64X && v == SEM_AX_OTF_SCALE)
@@ -807,6 +812,8 @@ sem_status cg_alloc(sem_mesh m, sem_prec prec, sem_ax_variant v, int precond, do
 sem_status cached_cg(sem_mesh m, sem_prec prec, sem_ax_variant v, int precond, int use_graph, double rtol,
                      int max_iter, sem_cg* out) {
   sem_cg& slot = prec == SEM_F32 ? m->solve_cg32 : m->solve_cg64;
+  int shape;
+  resolve_variant(m, prec, v, &v, &shape);
   if (slot && (slot->prec != prec || slot->variant != v || slot->precond != precond || slot->use_graph != use_graph)) {
     cg_free(slot);
     slot = nullptr;
@@ -839,10 +846,11 @@ sem_status cg_start(sem_cg c, const void* b, void* x, bool x0_is_zero, cudaStrea
     // The residual of a (re)start is formed with the native FP64 operator also when the
     // iterations run in double-float arithmetic: a restart after the recursive residual has
     // converged then replaces it by the true residual b - A x, and the solve corrects the
-    // double-float operator's own rounding (about 1e-14 of |A| |x|) instead of stalling on it.
+    // double-float operator's own rounding (about 1e-14 of |A| |x|) instead of stalling on it. (Where
+    // f64x_on_slices both are the same operator.)
     sem_prec rp = c->prec;
     sem_ax_variant rv = c->variant;
-    if (rp == SEM_F64X) {
+    if (rp == SEM_F64X && !(rv == SEM_AX_STORED && f64x_on_slices(m->N))) {
       rp = SEM_F64;
       if (rv == SEM_AX_STORED && !has_factors(m, SEM_F64)) rv = SEM_AX_OTF;
     }
@@ -864,7 +872,7 @@ AxLaunch cg_ax_launch(sem_cg c) {
   a.w = c->w;
   a.z = c->z;
   a.p = c->p;
-  if (fused_cg(c->prec)) {
+  if (cg_fused(c)) {
     a.r = c->r;
     a.minv = minv_of(c);
     a.x = c->x;
@@ -883,13 +891,13 @@ sem_status cg_enqueue_gs(sem_cg c, cudaStream_t s) {
 }
 
 sem_status cg_enqueue_update(sem_cg c, cudaStream_t s) {
-  return launch_cg_update(data_prec(c->prec), fused_cg(c->prec), c->m->n, c->x, c->p, c->r, c->w, c->z, minv_of(c),
+  return launch_cg_update(data_prec(c->prec), cg_fused(c), c->m->n, c->x, c->p, c->r, c->w, c->z, minv_of(c),
                           c->m->mult, c->m->ctab, c->st, c->upd_part, c->m->cg_map, s);
 }
 
 // fused_cg: the x update of the last iteration run (a no-op if there is none)
 sem_status cg_enqueue_flush(sem_cg c, cudaStream_t s) {
-  if (!fused_cg(c->prec)) return SEM_OK;
+  if (!cg_fused(c)) return SEM_OK;
   return launch_cg_flush(data_prec(c->prec), c->m->n, c->x, c->p, c->st, s);
 }
 
@@ -973,7 +981,7 @@ sem_status cg_iterate(sem_cg c, int k, cudaStream_t s) {
     c->exec_x = c->x;
   }
   SEM_CUDA_TRY(cudaGraphLaunch(c->exec, s));
-  count_launch(3 * k + (fused_cg(c->prec) ? 1 : 0));
+  count_launch(3 * k + (cg_fused(c) ? 1 : 0));
   return SEM_OK;
 }
 

@@ -28,9 +28,10 @@
 // as integers and rounded to FP64 once.
 //
 // What bounds it: GB300's integer instructions, 64 a clock per SM whatever their kind, with the
-// mma.sync and FP32 ones beside them (365 instructions per point, 46% of the issue slots, 0.43 of
+// mma.sync and FP32 ones beside them (about 360 instructions per point, 46% of the issue slots, 0.46 of
 // the HBM time). 16.8M points, N = 7: 1.502 ms in FP64 (k_ax, 95% of the FP64 peak by Eq. 11 flops) ->
-// 0.36 ms; in CG mode 1.562 -> 0.394 ms, one Jacobi-CG iteration 1.793 -> 0.624 ms.
+// 0.344 ms. In CG mode with the fused prologue 0.414 ms; it takes 0.02 ms from the operator's earlier
+// unfused form (0.394) and saves 0.067 in the update kernel: one Jacobi-CG iteration 1.793 -> 0.578 ms.
 //
 // Error against 64 bits (relative 2-norm of w, N = 7, jittered elements, CPU model of both
 // kernels against an 80-bit reference; k_ax in brackets): random u 8e-17 (1.8e-16), a sine over 8^3
@@ -302,13 +303,17 @@ struct Acc2 {  // (sum xh vh, sum xh vl + xl vh)
   __device__ __forceinline__ long long value() const { return h + (m >> 32); }
 };
 
-// 2^k for -1022 <= k <= 1023.
-__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
-
-__device__ __forceinline__ double to_double(long long v) {
-  const double dh = __hiloint2double(0x45300000, static_cast<int>(static_cast<uint32_t>(v >> 32) ^ 0x80000000u));
-  const double dl = __hiloint2double(0x43300000, static_cast<int>(static_cast<uint32_t>(v)));
-  return (dh - 19342822341709703277445120.0 /* 2^84 + 2^63 + 2^52 */) + dl;
+// v 2^k rounded to nearest (|v| < 2^62, the result a normal number or zero), on the integer pipes: three
+// FP64 instructions per point would keep the FP64 pipe busy for a quarter of the kernel's time.
+__device__ __forceinline__ double to_double(long long v, int k) {
+  const long long s = v >> 63;
+  const unsigned long long a = static_cast<unsigned long long>((v ^ s) - s);
+  const uint32_t hi = static_cast<uint32_t>(a >> 32);
+  const int lz = hi ? __clz(static_cast<int>(hi)) : 32 + __clz(static_cast<int>(static_cast<uint32_t>(a)));
+  const unsigned long long m = ((a << (lz - 1)) + 512ull) >> 10;  // significand in bits 52..0 (2^53 when rounded up)
+  const uint32_t h = static_cast<uint32_t>(m >> 32) + (static_cast<uint32_t>(1023 + 62 - (lz - 1) + k - 1) << 20);
+  const uint32_t sign = static_cast<uint32_t>(static_cast<unsigned long long>(v) >> 32) & 0x80000000u;
+  return a ? __hiloint2double(static_cast<int>(h | sign), static_cast<int>(static_cast<uint32_t>(m))) : 0.0;
 }
 
 // The element in FP64, as k_ax computes it (lines through the even/odd split of D): w of the whole
@@ -393,7 +398,8 @@ __device__ __forceinline__ unsigned over_element(unsigned v, F&& op) {
 // A block takes a group of kElems elements as one 8 x 8 x 8 box of points (one element for NP > 4).
 // Warp q holds the points of planes k = 2q and 2q + 1, lane (j = lane / 4, i = 2 (lane % 4) + {0, 1}), both
 // of one element; lanes and planes beyond an element's points hold zeros. Phases of a group:
-//   0  u (CG: p = z + beta p) to registers; largest exponent; digits of U to shared memory
+//   0  u (CG, fused_cg: the previous iteration's x += alpha p, p = M^-1 r + beta p) to registers; largest
+//      exponent; digits of U to shared memory
 //   1  k-lines (a warp takes j = 2q, 2q + 1): ut, exchanged through shared memory; i-rows and j-lines
 //      of the own planes: ur, us stay in the lane that owns the point; largest magnitude
 //   2  geometry; digits of vt to shared memory
@@ -404,8 +410,9 @@ template <int NP, bool CG>
 __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
     k_ax_slice(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab sl, int64_t E,
                const double* __restrict__ u, double* __restrict__ w, const int2* __restrict__ G,
-               const int* __restrict__ gexp, const double* __restrict__ z, double* __restrict__ p,
-               CgScalars* __restrict__ st, double* __restrict__ partials, int* __restrict__ err) {
+               const int* __restrict__ gexp, const double* __restrict__ r, const double* __restrict__ minv,
+               double* __restrict__ x, double* __restrict__ p, CgScalars* __restrict__ st,
+               double* __restrict__ partials, int* __restrict__ err) {
   using S = SliceShape<NP>;
   constexpr int NP2 = NP * NP, P = NP2 * NP, PL = S::kPlane;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -418,10 +425,11 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + S::kOffBar);
   __shared__ double sRed[32];
 
-  double beta = 0.0;
+  double beta = 0.0, alpha = 0.0;
   if constexpr (CG) {
     if (st->done) return;  // uniform over the grid: set by an earlier launch
     beta = st->beta;
+    alpha = st->alpha;
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int j = lane >> 2, i0 = 2 * (lane & 3), k0 = 2 * warp;
@@ -520,17 +528,23 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
     // phase 0
     double v[2][2];
     if constexpr (CG) {
-      double zv[2][2], pv[2][2];
+      double rv[2][2], pv[2][2], xv[2][2], mv[2][2];
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
-        load2(z, t, zv[t]);
+        load2(r, t, rv[t]);
         load2(p, t, pv[t]);
+        load2(x, t, xv[t]);
+        if (minv) load2(minv, t, mv[t]);
       }
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
 #pragma unroll
-        for (int x = 0; x < 2; ++x) v[t][x] = zv[t][x] + beta * pv[t][x];
+        for (int q = 0; q < 2; ++q) {
+          v[t][q] = fma(beta, pv[t][q], minv ? mv[t][q] * rv[t][q] : rv[t][q]);
+          xv[t][q] = fma(alpha, pv[t][q], xv[t][q]);
+        }
         store2(p, t, v[t]);
+        store2(x, t, xv[t]);
       }
     } else {
 #pragma unroll
@@ -562,8 +576,10 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
         const int64_t at = (e0 + static_cast<int64_t>(gridDim.x) * S::kElems) * P;
         const unsigned bytes = 8u * P * group_size(grp + gridDim.x);
         if constexpr (CG) {
-          l2_prefetch(z + at, bytes);
+          l2_prefetch(r + at, bytes);
           l2_prefetch(p + at, bytes);
+          l2_prefetch(x + at, bytes);
+          if (minv) l2_prefetch(minv + at, bytes);
         } else {
           l2_prefetch(u + at, bytes);
         }
@@ -730,12 +746,12 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
       }
       __syncthreads();
       // w = sum 2^-sc: u 2^(1080 - emax), D 2^e / 2^57 twice, V 2^lv, G 2^sg / 2^64
-      const double scale = pow2(-(1080 - emax + lv + sg - 64 + 2 * (sl.e - 57)));
+      const int scale = -(1080 - emax + lv + sg - 64 + 2 * (sl.e - 57));
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
         const longlong2 r = *reinterpret_cast<const longlong2*>(sX + (k0 + t) * PL + j * 8 + i0);
-        wv[t][0] = to_double(sum[t][0] + r.x) * scale;
-        wv[t][1] = to_double(sum[t][1] + r.y) * scale;
+        wv[t][0] = to_double(sum[t][0] + r.x, scale);
+        wv[t][1] = to_double(sum[t][1] + r.y, scale);
       }
     } else {
       for (int q = 0; q < S::kElems && e0 + q < E; ++q)
@@ -789,7 +805,8 @@ sem_status launch_slice_t(int N, const AxLaunch& a, cudaStream_t s) {
   if (a.grid_out) *a.grid_out = grid;
   k_ax_slice<NP, CG><<<grid, S::kThreads, S::kBytes, s>>>(
       tab, sl, a.E, static_cast<const double*>(a.u), static_cast<double*>(a.w), static_cast<const int2*>(a.G), a.gexp,
-      static_cast<const double*>(a.z), static_cast<double*>(a.p), a.st, a.partials, a.err);
+      static_cast<const double*>(a.r), static_cast<const double*>(a.minv), static_cast<double*>(a.x),
+      static_cast<double*>(a.p), a.st, a.partials, a.err);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;

@@ -156,7 +156,9 @@ __global__ void __launch_bounds__(SmallCg<NP>::kThreads, 1)
         for (int k = 0; k < NP; ++k) {
           if ((k < K2) != (h == 0)) continue;
           const int64_t q = eb + k * NP2 + t;
-          const double v = z[q] + beta * p[q];
+          // (z formed from r where the three-kernel path does so too and keeps no z, see cg_fused)
+          const double zq = !ax_slice_order(NP - 1) ? z[q] : minv ? minv[q] * r[q] : r[q];
+          const double v = zq + beta * p[q];
           p[q] = v;
           sA[Stage<NP>::at(la, lb, k)] = v;
         }

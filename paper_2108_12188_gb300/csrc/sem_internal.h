@@ -141,7 +141,11 @@ inline int64_t factor_stride(int Np, bool fp32) {
 // the 8 x 8 x 8 points a block works on (0.86 against 0.93 ms, 1.13 against 1.31). At N = 1 the FP64
 // differences of equal values are exact zeros, which fixed-point factors do not keep on stretched
 // elements (relative error 1.4e-15 against 1.2e-16 at aspect ratio 100).
-constexpr bool ax_slice_order(int N) { return N == 3 || N == 5 || N == 6 || N == 7; }
+__host__ __device__ constexpr bool ax_slice_order(int N) { return N == 3 || N == 5 || N == 6 || N == 7; }
+// SEM_F64X with stored factors runs there too at N = 7: it is the faster of the two and the more accurate
+// (A_L 0.344 against 0.409 ms in double-float at 16.8M points, a CG iteration 0.578 against 0.643; N = 3 0.36
+// against 0.27, N = 5 0.79 against 0.38, N = 6 0.62 against 0.50).
+__host__ __device__ constexpr bool f64x_on_slices(int N) { return N == 7; }
 __host__ __device__ constexpr int fixed_row_scale(int NP, int i) {
   return i == 0 || i == NP - 1 ? (NP <= 4 ? 1 : 2) : 0;
 }
@@ -236,10 +240,10 @@ struct sem_mesh_s {
   double* coef64 = nullptr;   // [E][24] trilinear coefficients a0..a7 (x, y, z)
   float* coef32 = nullptr;    // [E][24] rounded to FP32
   double* G64 = nullptr;      // [E][6][P] or null (ax_slice_order: only for fewer elements than SMs)
-  int2* GI = nullptr;         // [E][6][P] fixed-point factors (ax_slice_order) or null
+  int2* GI = nullptr;         // [E][6][P] fixed-point factors (ax_slice_order; at N = 7 for SEM_F64X too) or null
   int* gexp = nullptr;        // [E] their exponents sg
   float* G32 = nullptr;       // [E][factor_stride] (the [6][P] block, padded to 16 bytes) or null
-  float* Gx = nullptr;        // [E][6][P] float pairs (high, low) of G for SEM_F64X, or null
+  float* Gx = nullptr;        // [E][6][P] float pairs (high, low) of G for SEM_F64X (but f64x_on_slices), or null
   double* scale64 = nullptr;  // [n] w_i w_j w_k / det J (SEM_MESH_OTF_SCALE) or null
   float* scale32 = nullptr;
   int32_t* gs_rec[sem::kGsClasses] = {};  // gather-scatter plan (views in gs)
@@ -294,7 +298,7 @@ struct AxLaunch {
   // CG mode (p = z + beta p prologue, <p, w> partials in the epilogue)
   const void* z;
   void* p;
-  // fused CG prologue (FP32 and double-float operators, fused_cg): x += alpha p, the update
+  // fused CG prologue (fused_cg): x += alpha p, the update
   // deferred from the previous iteration, and z = M^-1 r (minv null: no preconditioner)
   const void* r;
   const void* minv;
@@ -389,9 +393,12 @@ inline bool whole_dot(sem_prec) { return true; }  // every CG-mode operator form
 // fit in L2 and the gather-scatter is bound by DRAM sectors. FP32 CG keeps the local layout (its
 // w stays in L2, and reading w through the map costs the FP32 update more than it saves).
 inline bool cg_layout(sem_prec prec) { return prec != SEM_F32; }
-// The same operators take the fused CG prologue (AxLaunch::r, minv, x): the update kernel
-// then skips x and z, and after the last iteration launch_cg_flush adds the pending alpha p.
-inline bool fused_cg(sem_prec prec) { return prec != SEM_F64; }
+// The FP32, double-float and tensor-core FP64 operators take the fused CG prologue (AxLaunch::r, minv,
+// x): the update kernel then skips x and z, and after the last iteration launch_cg_flush adds the
+// pending alpha p. The FP64-pipe-bound k_ax leaves both to the update kernel.
+inline bool fused_cg(sem_prec prec, int N, sem_ax_variant v) {
+  return prec != SEM_F64 || (v == SEM_AX_STORED && ax_slice_order(N));
+}
 sem_status launch_dssum_cg(sem_prec prec, const GsPlan& g, void* w, const void* p, CgScalars* st,
                            const double* ax_partials, int ax_blocks, double* partials, cudaStream_t s);
 // Batched kernels (k_batch.cu) over the device table `t` (host copy `h` gives the orders present
