@@ -710,7 +710,7 @@ struct sem_cg_s {
   const void* b = nullptr;
   CgScalars* st = nullptr;
   CgScalars st_host{};  // host mirror of the device scalars (pageable: no device-wide synchronisation)
-  double *ax_part = nullptr, *gs_part = nullptr, *upd_part = nullptr, *init_part = nullptr;
+  double *ax_part = nullptr, *upd_part = nullptr, *init_part = nullptr;
   int ax_blocks = 0;
   cudaStream_t cap = nullptr;     // private stream: allocation, graph capture, release
   unsigned* bar = nullptr;        // grid barrier words of the persistent small-mesh kernel
@@ -744,7 +744,6 @@ void cg_free(sem_cg c) {
   for (void* q : {c->r, c->z, c->p, c->w})
     if (q) cudaFreeAsync(q, h);
   dfree(c->ax_part, h);
-  dfree(c->gs_part, h);
   dfree(c->upd_part, h);
   dfree(c->init_part, h);
   dfree(c->st, h);
@@ -793,7 +792,6 @@ sem_status cg_alloc(sem_mesh m, sem_prec prec, sem_ax_variant v, int precond, do
     }
   }
   if (st == SEM_OK) st = dmalloc(&c->ax_part, kRedMax, nullptr, c->cap);
-  if (st == SEM_OK) st = dmalloc(&c->gs_part, kRedMax, nullptr, c->cap);
   if (st == SEM_OK) st = dmalloc(&c->upd_part, 2 * kRedMax, nullptr, c->cap);
   if (st == SEM_OK) st = dmalloc(&c->init_part, 3 * kRedMax, nullptr, c->cap);
   if (st == SEM_OK) st = dmalloc(&c->st, 1, nullptr, c->cap);
@@ -883,11 +881,10 @@ AxLaunch cg_ax_launch(sem_cg c) {
   return a;
 }
 
-// QQ^T and the mask on w (FP64 data: in the CG layout); every CG-mode operator formed the whole
-// <p, w>.
+// QQ^T and the mask on w (FP64 data: in the CG layout), and alpha from the operator's <p, w>.
 sem_status cg_enqueue_gs(sem_cg c, cudaStream_t s) {
-  return launch_dssum_cg(data_prec(c->prec), cg_layout(c->prec) ? c->m->gs_cg : c->m->gs, c->w,
-                         whole_dot(c->prec) ? nullptr : c->p, c->st, c->ax_part, c->ax_blocks, c->gs_part, s);
+  return launch_dssum_cg(data_prec(c->prec), cg_layout(c->prec) ? c->m->gs_cg : c->m->gs, c->w, c->st, c->ax_part,
+                         c->ax_blocks, s);
 }
 
 sem_status cg_enqueue_update(sem_cg c, cudaStream_t s) {
@@ -901,8 +898,7 @@ sem_status cg_enqueue_flush(sem_cg c, cudaStream_t s) {
   return launch_cg_flush(data_prec(c->prec), c->m->n, c->x, c->p, c->st, s);
 }
 
-// One iteration of Algorithm 1: [p = z + beta p; w = A_L p; <p,w> partials] -> [QQ^T, mask,
-// (boundary <p,w>), alpha] -> [r, z (and x) updates, <r,z,c>, <r,r,c>, beta, stop test].
+// One iteration of Algorithm 1: [p = z + beta p; w = A_L p; <p,w> partials] -> [QQ^T, mask, alpha] -> [r, z (and x) updates, <r,z,c>, <r,r,c>, beta, stop test].
 sem_status cg_enqueue_iteration(sem_cg c, cudaStream_t s) {
   SEM_TRY(launch_ax_any(c->m, c->prec, c->variant, true, cg_ax_launch(c), s));
   SEM_TRY(cg_enqueue_gs(c, s));

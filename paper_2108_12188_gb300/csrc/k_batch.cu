@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(NP * NP * EPB)
   using F = float;
   constexpr int NP2 = NP * NP, P = NP2 * NP, SZ = Stage<NP>::kSize;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ double sRed[32];
+  __shared__ double sRed[NP * NP * EPB];
   F* sA0 = reinterpret_cast<F*>(smem_raw);
   F* sB0 = sA0 + EPB * SZ;
   const BatchOrder ord = T->order[NP];
@@ -146,8 +146,7 @@ __global__ void __launch_bounds__(NP * NP * EPB)
     }
     __syncthreads();
     // phase 5: w on the column, and this group's part of <p, w> (over every point; the column
-    // as one multiply-add chain, added to a compensated sum)
-    DotAcc<F> dot;
+    // as one multiply-add chain)
     F* __restrict__ w = d->w;
     F col = F(0);
 #pragma unroll
@@ -157,10 +156,10 @@ __global__ void __launch_bounds__(NP * NP * EPB)
       if (valid) w[base + k * NP2] = acc;
       col = fmaf(rU[k], acc, col);
     }
-    if (valid) dot.add_sum(col);
-    // (block_sum's barriers also keep the staging buffers until every thread has read them)
-    const double s = block_sum(dot.value(), sRed);
-    if (threadIdx.x == 0) d->ax_part[grp] = s;
+    // (block_sums' barriers also keep the staging buffers until every thread has read them)
+    double s[1] = {valid ? fp64_of(col) : 0.0};
+    block_sums<1, NP * NP * EPB>(s, sRed);
+    if (threadIdx.x == 0) d->ax_part[grp] = s[0];
   }
 }
 
@@ -181,11 +180,10 @@ __device__ __forceinline__ void gs_chunk(const int32_t* __restrict__ rec, const 
   }
 }
 
-// Algorithm 1 step 7 (QQ^T and the mask) for every solve; the item that completes a solve
-// forms <p, w, c> from the operator's group partials and alpha = rho / <p, w, c> (step 8).
+// Algorithm 1 step 7 (QQ^T and the mask) for every solve; a solve's first item also adds the operator's
+// group partials (complete at this launch) to <p, w, c> and forms alpha = rho / <p, w, c> (step 8).
 __global__ void __launch_bounds__(kBatchThreads) k_gs_batch(const BatchTable* __restrict__ T) {
-  __shared__ double sRed[kBatchThreads / 32];
-  __shared__ bool last;
+  __shared__ double sRed[kBatchThreads];
   const int64_t items = T->gs_items;
   int sv = 0;
   for (int64_t q = blockIdx.x; q < items; q += gridDim.x) {
@@ -215,25 +213,17 @@ __global__ void __launch_bounds__(kBatchThreads) k_gs_batch(const BatchTable* __
         }
       }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      const unsigned t = atomicAdd(&st->ticket[0], 1u);
-      last = t == static_cast<unsigned>(d->gs_at[5] - 1);
-      if (last) st->ticket[0] = 0u;
-    }
-    __syncthreads();
-    if (last) {
-      __threadfence();
-      const double pw = sum_partials(d->ax_part, static_cast<int>(d->ax_cnt), 1, 0, sRed);
+    if (l == 0) {
+      double pw[1];
+      partial_sums<1, kBatchThreads>(d->ax_part, static_cast<int>(d->ax_cnt), pw, sRed);
       if (threadIdx.x == 0) {
-        st->pw = pw;
-        if (!(pw > 0.0) || !isfinite(pw)) {
+        st->pw = pw[0];
+        if (!(pw[0] > 0.0) || !isfinite(pw[0])) {
           st->status = SEM_ERR_BREAKDOWN;
           st->done = 1;
           st->alpha = 0.0;
         } else {
-          st->alpha = st->rho / pw;
+          st->alpha = st->rho / pw[0];
         }
       }
     }
@@ -244,9 +234,13 @@ __global__ void __launch_bounds__(kBatchThreads) k_gs_batch(const BatchTable* __
 // partials of <r, z, c> and <r, r, c> per chunk; the item that completes a solve forms rho,
 // beta, the iteration count and the stopping decision.
 __global__ void __launch_bounds__(kBatchThreads) k_update_batch(const BatchTable* __restrict__ T) {
-  __shared__ double sRed[kBatchThreads / 32];
+  __shared__ double sRed[2 * kBatchThreads];
+  __shared__ float sC[256];  // c = 1 / multiplicity, the same table for every mesh
   __shared__ bool last;
   const int64_t items = T->up_items;
+  if (blockIdx.x >= items) return;
+  for (int m = threadIdx.x; m < 256; m += kBatchThreads) sC[m] = m == 1 ? 1.f : static_cast<float>(T->s[0].ctab[m]);
+  __syncthreads();
   int sv = 0;
   for (int64_t q = blockIdx.x; q < items; q += gridDim.x) {
     while (q >= T->s[sv].up_beg + T->s[sv].up_cnt) ++sv;
@@ -261,12 +255,11 @@ __global__ void __launch_bounds__(kBatchThreads) k_update_batch(const BatchTable
     const float* __restrict__ w = d->w;
     const float* __restrict__ minv = d->minv;
     const uint8_t* __restrict__ mult = d->mult;
-    const double* __restrict__ ctab = d->ctab;
     DotAcc<float> rz, rr;
     auto point = [&](float& ri, float wi, float mi, unsigned m) {
       ri = ri - alpha * wi;
       const float zi = minv ? mi * ri : ri;
-      const float cw = m == 1u ? 1.f : static_cast<float>(__ldg(ctab + m));
+      const float cw = sC[m];
       rz.add(ri, cw * zi);
       rr.add(ri, cw * ri);
     };
@@ -297,11 +290,11 @@ __global__ void __launch_bounds__(kBatchThreads) k_update_batch(const BatchTable
         r[i] = ri;
       }
     }
-    const double vz = block_sum(rz.value(), sRed);
-    const double vr = block_sum(rr.value(), sRed);
+    double v[2] = {rz.value(), rr.value()};
+    block_sums<2, kBatchThreads>(v, sRed);
     if (threadIdx.x == 0) {
-      d->up_part[2 * c] = vz;
-      d->up_part[2 * c + 1] = vr;
+      d->up_part[2 * c] = v[0];
+      d->up_part[2 * c + 1] = v[1];
       __threadfence();
       const unsigned t = atomicAdd(&st->ticket[1], 1u);
       last = t == static_cast<unsigned>(d->up_cnt - 1);
@@ -311,8 +304,8 @@ __global__ void __launch_bounds__(kBatchThreads) k_update_batch(const BatchTable
     if (last) {
       __threadfence();
       const int cnt = static_cast<int>(d->up_cnt);
-      const double srz = sum_partials(d->up_part, cnt, 2, 0, sRed);
-      const double srr = sum_partials(d->up_part, cnt, 2, 1, sRed);
+      partial_sums<2, kBatchThreads>(d->up_part, cnt, v, sRed);
+      const double srz = v[0], srr = v[1];
       if (threadIdx.x == 0) {
         const int it = st->iter + 1;
         st->iter = it;

@@ -69,7 +69,7 @@ template <typename T>
 __global__ void k_glsc3(int64_t n, const T* __restrict__ a, const T* __restrict__ b, const uint8_t* __restrict__ mult,
                         const double* __restrict__ ctab, double* __restrict__ partials, unsigned int* ticket,
                         double* __restrict__ result) {
-  __shared__ double sRed[kThreads / 32];
+  __shared__ double sRed[kThreads];
   double acc = 0.0;
   const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -102,10 +102,11 @@ __global__ void k_glsc3(int64_t n, const T* __restrict__ a, const T* __restrict_
     }
   }
   for (int64_t i = 4 * n4 + t0; i < n; i += stride) general(a[i], b[i], mult[i]);
-  const double v[1] = {block_sum(acc, sRed)};
+  double v[1] = {acc};
+  block_sums<1, kThreads>(v, sRed);
   if (publish_partials<1>(v, partials, ticket)) {
-    const double s = sum_partials(partials, gridDim.x, 1, 0, sRed);
-    if (threadIdx.x == 0) *result = s;
+    partial_sums<1, kThreads>(partials, gridDim.x, v, sRed);
+    if (threadIdx.x == 0) *result = v[0];
   }
 }
 
@@ -116,7 +117,7 @@ __global__ void k_cg_init(int64_t n, const T* __restrict__ b, const T* __restric
                           T* __restrict__ z, T* __restrict__ p, const T* __restrict__ minv,
                           const uint8_t* __restrict__ mult, const double* __restrict__ ctab, CgScalars* st,
                           double* __restrict__ partials) {
-  __shared__ double sRed[kThreads / 32];
+  __shared__ double sRed[3 * kThreads];
   DotAcc<T> rz, rr, bb;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -131,11 +132,11 @@ __global__ void k_cg_init(int64_t n, const T* __restrict__ b, const T* __restric
     rr.add(ri, c * ri);
     bb.add(bi, c * bi);
   }
-  const double v[3] = {block_sum(rz.value(), sRed), block_sum(rr.value(), sRed), block_sum(bb.value(), sRed)};
+  double v[3] = {rz.value(), rr.value(), bb.value()};
+  block_sums<3, kThreads>(v, sRed);
   if (publish_partials<3>(v, partials, &st->ticket[2])) {
-    const double srz = sum_partials(partials, gridDim.x, 3, 0, sRed);
-    const double srr = sum_partials(partials, gridDim.x, 3, 1, sRed);
-    const double sbb = sum_partials(partials, gridDim.x, 3, 2, sRed);
+    partial_sums<3, kThreads>(partials, gridDim.x, v, sRed);
+    const double srz = v[0], srr = v[1], sbb = v[2];
     if (threadIdx.x == 0) {
       st->rho = srz;
       st->rz = srz;
@@ -183,12 +184,15 @@ struct Vec16<float> {
 // operator in the CG layout and assembled there by the gather-scatter, is read through `map`.
 // FUSED: the operator's CG prologue makes x += alpha p (one iteration later) and recomputes
 // z = M^-1 r, so this kernel leaves x alone and stores no z (z is formed for the dots only).
+// 16.8M points, fused: FP64 data 106 us (HBM time 82). At small sizes a launch is a chain of latencies,
+// of which the FP64 instructions of the block sums and of the FP32 weights' conversions were the largest
+// part: 371k FP32 points 16.4 -> 10.4 us with block_sums, the weights from a table and half the blocks.
 template <typename T, bool FUSED>
-__global__ void k_cg_update(int64_t n, T* __restrict__ x, const T* __restrict__ p, T* __restrict__ r,
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 5 : 4) k_cg_update(int64_t n, T* __restrict__ x, const T* __restrict__ p, T* __restrict__ r,
                             const T* __restrict__ w, T* __restrict__ z, const T* __restrict__ minv,
                             const uint8_t* __restrict__ mult, const double* __restrict__ ctab, CgScalars* st,
                             double* __restrict__ partials, const CgMap map) {
-  __shared__ double sRed[kThreads / 32];
+  __shared__ double sRed[2 * kThreads];  // the weights' table, then the block's sums
   if (st->done) return;
   using VT = typename Vec16<T>::type;
   using MT = typename Vec16<T>::mtype;
@@ -280,7 +284,7 @@ __global__ void k_cg_update(int64_t n, T* __restrict__ x, const T* __restrict__ 
     // product term is kept: cut off, they shift both sums by about 1e-14 the same way at every
     // point, and with them alpha and beta (x after 10 iterations on 8^3 elements: 5.1e-14 off a long-double
     // computation with the cut-off, 3.9e-15 without, in the same time).
-    __shared__ df2 sC[256];
+    df2* sC = reinterpret_cast<df2*>(sRed);
     for (int m = threadIdx.x; m < 256; m += blockDim.x) sC[m] = m == 1 ? df2{1.f, 0.f} : df_split<true>(ctab[m]);
     __syncthreads();
     df2 rz{0.f, 0.f}, rr{0.f, 0.f};
@@ -294,24 +298,30 @@ __global__ void k_cg_update(int64_t n, T* __restrict__ x, const T* __restrict__ 
       df_fma_acc_full(rz, ch, cl, z2.h, z2.l);
       df_fma_acc_full(rr, ch, cl, r2.h, r2.l);
     });
-    v[0] = block_sum(static_cast<double>(rz.h) + static_cast<double>(rz.l), sRed);
-    v[1] = block_sum(static_cast<double>(rr.h) + static_cast<double>(rr.l), sRed);
+    v[0] = fp64_of(rz.h) + fp64_of(rz.l);
+    v[1] = fp64_of(rr.h) + fp64_of(rr.l);
   } else {
+    // c from a table in shared memory: rounding the FP64 table's entry at every point is an FP64-pipe
+    // instruction per point
+    float* sC = reinterpret_cast<float*>(sRed);
+    for (int m = threadIdx.x; m < 256; m += blockDim.x) sC[m] = m == 1 ? 1.f : static_cast<float>(ctab[m]);
+    __syncthreads();
     DotAcc<T> rz, rr;
     sweep([&](T& xi, T pi, T& ri, T wi, T& zi, T mi, unsigned m) {
       if constexpr (!FUSED) xi += alpha * pi;
       ri = ri - alpha * wi;
       zi = minv ? mi * ri : ri;
-      const T c = m == 1u ? T(1) : static_cast<T>(__ldg(ctab + m));
+      const T c = sC[m];
       rz.add(ri, c * zi);
       rr.add(ri, c * ri);
     });
-    v[0] = block_sum(rz.value(), sRed);
-    v[1] = block_sum(rr.value(), sRed);
+    v[0] = rz.value();
+    v[1] = rr.value();
   }
+  block_sums<2, kThreads>(v, sRed);
   if (publish_partials<2>(v, partials, &st->ticket[1])) {
-    const double srz = sum_partials(partials, gridDim.x, 2, 0, sRed);
-    const double srr = sum_partials(partials, gridDim.x, 2, 1, sRed);
+    partial_sums<2, kThreads>(partials, gridDim.x, v, sRed);
+    const double srz = v[0], srr = v[1];
     if (threadIdx.x == 0) {
       const int it = st->iter + 1;
       st->iter = it;
@@ -373,9 +383,11 @@ sem_status launch_cg_init(sem_prec prec, int64_t n, const void* b, const void* a
 sem_status launch_cg_update(sem_prec prec, bool fused, int64_t n, void* x, const void* p, void* r, const void* w,
                             void* z, const void* minv, const uint8_t* mult, const double* ctab, CgScalars* st,
                             double* partials, const CgMap& map, cudaStream_t s) {
-  const int grid = vec_grid(n, prec != SEM_F64 ? resident_blocks<k_cg_update<float, true>>(kThreads)
-                               : fused         ? resident_blocks<k_cg_update<double, true>>(kThreads)
-                                               : resident_blocks<k_cg_update<double, false>>(kThreads));
+  // at least two 16-byte steps per thread: every block costs a reduction and a ticket
+  const int grid = vec_grid(n * (prec == SEM_F32 ? 4 : 8) / 32,
+                            prec != SEM_F64 ? resident_blocks<k_cg_update<float, true>>(kThreads)
+                            : fused         ? resident_blocks<k_cg_update<double, true>>(kThreads)
+                                            : resident_blocks<k_cg_update<double, false>>(kThreads));
   if (prec == SEM_F64) {
     auto* xd = static_cast<double*>(x);
     auto* pd = static_cast<const double*>(p);
@@ -447,7 +459,7 @@ namespace {
 __global__ void k_ir_residual(int64_t n, const double* __restrict__ b, const double* __restrict__ w,
                               double* __restrict__ r64, float* __restrict__ r32, const uint8_t* __restrict__ mult,
                               const double* __restrict__ ctab, CgScalars* st, double* __restrict__ partials) {
-  __shared__ double sRed[kThreads / 32];
+  __shared__ double sRed[2 * kThreads];
   double rr = 0.0, bb = 0.0;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -458,10 +470,11 @@ __global__ void k_ir_residual(int64_t n, const double* __restrict__ b, const dou
     rr += c * ri * ri;
     bb += c * bi * bi;
   }
-  const double v[2] = {block_sum(rr, sRed), block_sum(bb, sRed)};
+  double v[2] = {rr, bb};
+  block_sums<2, kThreads>(v, sRed);
   if (publish_partials<2>(v, partials, &st->ticket[3])) {
-    const double srr = sum_partials(partials, gridDim.x, 2, 0, sRed);
-    const double sbb = sum_partials(partials, gridDim.x, 2, 1, sRed);
+    partial_sums<2, kThreads>(partials, gridDim.x, v, sRed);
+    const double srr = v[0], sbb = v[1];
     if (threadIdx.x == 0) {
       st->rr = srr;
       st->bb = sbb;
@@ -484,7 +497,7 @@ __global__ void k_ir_residual(int64_t n, const double* __restrict__ b, const dou
 __global__ void k_cg_replace(int64_t n, const float* __restrict__ rnew, float* __restrict__ r, float* __restrict__ z,
                              const float* __restrict__ minv, const uint8_t* __restrict__ mult,
                              const double* __restrict__ ctab, CgScalars* st, double* __restrict__ partials) {
-  __shared__ double sRed[kThreads / 32];
+  __shared__ double sRed[2 * kThreads];
   DotAcc<float> rz, rr;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -496,10 +509,11 @@ __global__ void k_cg_replace(int64_t n, const float* __restrict__ rnew, float* _
     rz.add(ri, c * zi);
     rr.add(ri, c * ri);
   }
-  const double v[2] = {block_sum(rz.value(), sRed), block_sum(rr.value(), sRed)};
+  double v[2] = {rz.value(), rr.value()};
+  block_sums<2, kThreads>(v, sRed);
   if (publish_partials<2>(v, partials, &st->ticket[2])) {
-    const double srz = sum_partials(partials, gridDim.x, 2, 0, sRed);
-    const double srr = sum_partials(partials, gridDim.x, 2, 1, sRed);
+    partial_sums<2, kThreads>(partials, gridDim.x, v, sRed);
+    const double srz = v[0], srr = v[1];
     if (threadIdx.x == 0) {
       if (!isfinite(srz) || !isfinite(srr) || !(st->rho > 0.0)) {
         st->status = SEM_ERR_BREAKDOWN;

@@ -137,6 +137,62 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return s;
 }
 
+// FP32 to FP64 by moving the fields where the value is normal or zero: the conversion instruction
+// runs on the FP64 pipe, which takes 64 cycles of a scheduler for a warp.
+__device__ __forceinline__ double fp64_of(float a) {
+  const unsigned u = __float_as_uint(a), mag = u & 0x7fffffffu;
+  if (mag - 0x00800000u < 0x7f000000u || mag == 0u) {
+    const unsigned hi = mag == 0u ? 0u : (mag >> 3) + (896u << 20);
+    return __hiloint2double(static_cast<int>((u & 0x80000000u) | hi), static_cast<int>(u << 29));
+  }
+  double d;
+  asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(a));  // volatile: not hoisted above the test
+  return d;
+}
+
+// Sums of K values over the T threads of the block in a fixed order, the results in every thread.
+// buf: K T doubles of shared memory. Warp q adds value q: with one value per thread in shared memory
+// that takes T / 32 + 4 FP64 instructions of one warp, where a shuffle tree in every warp (block_sum) takes
+// 5 T / 32 + T / 32. FP64 instructions keep a scheduler's FP64 pipe for 64 cycles each, so at small sizes
+// the block sums were most of a reducing kernel's time.
+template <int K, int T>
+__device__ __forceinline__ void block_sums(double (&v)[K], double* buf) {
+  constexpr int W = (T + 31) / 32;
+  static_assert(K <= T / 32, "one full warp per value");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < K; ++q) buf[q * T + tid] = v[q];
+  __syncthreads();
+  if (warp < K) {
+    double a[W];
+#pragma unroll
+    for (int r = 0; r < W; ++r) a[r] = T % 32 == 0 || r * 32 + lane < T ? buf[warp * T + r * 32 + lane] : 0.0;
+#pragma unroll
+    for (int d = 1; d < W; d *= 2)
+#pragma unroll
+      for (int r = 0; r + d < W; r += 2 * d) a[r] += a[r + d];
+    double s = a[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) buf[warp * T] = s;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < K; ++q) v[q] = buf[q * T];
+}
+
+// Fixed-order sums over q in [0, count) of partials[K q + c], c < K, in every thread.
+template <int K, int T>
+__device__ __forceinline__ void partial_sums(const double* partials, int count, double (&v)[K], double* buf) {
+#pragma unroll
+  for (int c = 0; c < K; ++c) v[c] = 0.0;
+  for (int q = threadIdx.x; q < count; q += T)
+#pragma unroll
+    for (int c = 0; c < K; ++c) v[c] += __ldcg(partials + K * q + c);
+  block_sums<K, T>(v, buf);
+}
+
 // Each block stores its partial(s); the block that arrives last (ticket) returns true
 // in every thread and may then read all partials. The ticket is reset for the next use.
 template <int K>
@@ -245,7 +301,7 @@ struct DotAcc<float> {
     hi = s;
     lo = __fadd_rn(lo, t);
   }
-  __device__ __forceinline__ double value() const { return static_cast<double>(hi) + static_cast<double>(lo); }
+  __device__ __forceinline__ double value() const { return fp64_of(hi) + fp64_of(lo); }
 };
 
 }  // namespace sem

@@ -44,11 +44,10 @@ __device__ __forceinline__ void for_class(const GsPlan& g, int c, int64_t t0, in
 
 // In-place gather-scatter of class c, two segments per thread at a time (both records, then
 // the copies of both, are loaded before anything is added or stored: segments never share
-// copies). value(masked, sum, pf) gives what is written to the copies; pf is pv at the
-// segment's first copy, loaded with the copies (0 if pv is null).
+// copies). value(masked, sum) gives what is written to the copies.
 template <int W, typename T, typename F>
 __device__ __forceinline__ void gs_class(const GsPlan& g, int c, int64_t t0, int64_t stride, T* __restrict__ u,
-                                         const T* __restrict__ pv, F&& value) {
+                                         F&& value) {
   const int64_t n = g.n[c];
   int64_t t = t0;
   for (; t + stride < n; t += 2 * stride) {
@@ -60,9 +59,8 @@ __device__ __forceinline__ void gs_class(const GsPlan& g, int c, int64_t t0, int
     T va[W], vb[W];
     seg_load<W>(u, a, va);
     seg_load<W>(u, b, vb);
-    const T pa = pv ? pv[a[0]] : T(0), pb = pv ? pv[b[0]] : T(0);
-    const T ra = value(ma, seg_add<W>(a, va), pa);
-    const T rb = value(mb, seg_add<W>(b, vb), pb);
+    const T ra = value(ma, seg_add<W>(a, va));
+    const T rb = value(mb, seg_add<W>(b, vb));
     seg_store<W>(u, a, ra);
     seg_store<W>(u, b, rb);
   }
@@ -72,8 +70,7 @@ __device__ __forceinline__ void gs_class(const GsPlan& g, int c, int64_t t0, int
     load_rec<W>(g.rec[c], s0, a);
     T va[W];
     seg_load<W>(u, a, va);
-    const T pa = pv ? pv[a[0]] : T(0);
-    seg_store<W>(u, a, value(g.msk[c][s0] != 0, seg_add<W>(a, va), pa));
+    seg_store<W>(u, a, value(g.msk[c][s0] != 0, seg_add<W>(a, va)));
   }
 }
 
@@ -81,11 +78,11 @@ template <typename T>
 __global__ void k_dssum(const GsPlan g, T* __restrict__ u, int apply_mask) {
   const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  auto value = [&](bool masked, T sum, T) { return (apply_mask && masked) ? T(0) : sum; };
-  gs_class<2>(g, 1, t0, stride, u, static_cast<const T*>(nullptr), value);
-  gs_class<4>(g, 2, t0, stride, u, static_cast<const T*>(nullptr), value);
-  gs_class<8>(g, 3, t0, stride, u, static_cast<const T*>(nullptr), value);
-  gs_class<1>(g, 0, t0, stride, u, static_cast<const T*>(nullptr), value);
+  auto value = [&](bool masked, T sum) { return (apply_mask && masked) ? T(0) : sum; };
+  gs_class<2>(g, 1, t0, stride, u, value);
+  gs_class<4>(g, 2, t0, stride, u, value);
+  gs_class<8>(g, 3, t0, stride, u, value);
+  gs_class<1>(g, 0, t0, stride, u, value);
   for (int64_t x = t0; x < g.nx; x += stride) {
     const int o0 = g.xoff[x], o1 = g.xoff[x + 1];
     T s = u[g.xidx[o0]];
@@ -95,74 +92,45 @@ __global__ void k_dssum(const GsPlan g, T* __restrict__ u, int apply_mask) {
   }
 }
 
-// CG step 7. DOT: also the boundary part of <p, w, c>: after the sum, all copies of a
-// segment hold the same w and the same p, and their weights c = 1/multiplicity add up to
-// one, so the segment contributes p * w once; the last block adds the operator's partials and
-// its own, forms <p, w, c> and alpha = rho / <p, w, c> (Algorithm 1 step 8). Without DOT the
-// operator has already formed the whole product over the unassembled w (sum over local points
-// of p_i (A_L p)_i equals <p, QQ^T A_L p, c> because p has one value per global node and is 0
-// on Dirichlet nodes): block 0 sums the operator's partials (complete at this launch) in a
-// fixed order and forms alpha before its share of the segments, and no block reduces anything
-// else (no ticket, no last block).
-template <typename T, bool DOT>
-__global__ void __launch_bounds__(kThreads, 4) k_dssum_cg(const GsPlan g, T* __restrict__ w, const T* __restrict__ p, CgScalars* __restrict__ st,
-                           const double* __restrict__ ax_partials, int ax_blocks, double* __restrict__ partials) {
-  __shared__ double sRed[kThreads / 32];
+// CG step 7, and alpha. The operator has formed <p, w, c> over the unassembled w (the sum over local points
+// of p_i (A_L p)_i equals <p, QQ^T A_L p, c> because p has one value per global node and is 0 on
+// Dirichlet nodes): block 0 adds its partials (complete at this launch) in a fixed order and forms
+// alpha = rho / <p, w, c> (Algorithm 1 step 8) while the other blocks take the segments, so the chain of
+// the sum and the division is not in front of any segment, and no block has a ticket or a last block's
+// work.
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 4) k_dssum_cg(const GsPlan g, T* __restrict__ w, CgScalars* __restrict__ st,
+                           const double* __restrict__ ax_partials, int ax_blocks) {
+  __shared__ double sRed[kThreads];
   if (st->done) return;
-  if constexpr (!DOT) {
-    if (blockIdx.x == 0) {
-      const double pw = sum_partials(ax_partials, ax_blocks, 1, 0, sRed);
-      if (threadIdx.x == 0) {
-        st->pw = pw;
-        if (!(pw > 0.0) || !isfinite(pw)) {
-          st->status = SEM_ERR_BREAKDOWN;
-          st->done = 1;
-          st->alpha = 0.0;  // x is not advanced along this p (fused CG: nothing left to flush)
-        } else {
-          st->alpha = st->rho / pw;
-        }
+  if (blockIdx.x == 0) {
+    double pw[1];
+    partial_sums<1, kThreads>(ax_partials, ax_blocks, pw, sRed);
+    if (threadIdx.x == 0) {
+      st->pw = pw[0];
+      if (!(pw[0] > 0.0) || !isfinite(pw[0])) {
+        st->status = SEM_ERR_BREAKDOWN;
+        st->done = 1;
+        st->alpha = 0.0;  // x is not advanced along this p (fused CG: nothing left to flush)
+      } else {
+        st->alpha = st->rho / pw[0];
       }
     }
+    return;
   }
-  const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  DotAcc<T> dot;
-  const T* pv = DOT ? p : nullptr;
-  auto value = [&](bool masked, T sum, T pf) {
-    const T s = masked ? T(0) : sum;
-    if constexpr (DOT) dot.add(pf, s);
-    return s;
-  };
-  gs_class<2>(g, 1, t0, stride, w, pv, value);
-  gs_class<4>(g, 2, t0, stride, w, pv, value);
-  gs_class<8>(g, 3, t0, stride, w, pv, value);
-  gs_class<1>(g, 0, t0, stride, w, pv, value);
+  const int64_t t0 = (blockIdx.x - 1) * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  const int64_t stride = static_cast<int64_t>(gridDim.x - 1) * blockDim.x;
+  auto value = [&](bool masked, T sum) { return masked ? T(0) : sum; };
+  gs_class<2>(g, 1, t0, stride, w, value);
+  gs_class<4>(g, 2, t0, stride, w, value);
+  gs_class<8>(g, 3, t0, stride, w, value);
+  gs_class<1>(g, 0, t0, stride, w, value);
   for (int64_t x = t0; x < g.nx; x += stride) {
     const int o0 = g.xoff[x], o1 = g.xoff[x + 1];
-    const int first = g.xidx[o0];
-    T s = w[first];
+    T s = w[g.xidx[o0]];
     for (int o = o0 + 1; o < o1; ++o) s += w[g.xidx[o]];
     if (g.xmsk[x]) s = T(0);
     for (int o = o0; o < o1; ++o) w[g.xidx[o]] = s;
-    if constexpr (DOT) dot.add(p[first], s);
-  }
-  if constexpr (DOT) {  // without DOT block 0 has formed alpha: nothing to reduce here
-    const double v[1] = {block_sum(dot.value(), sRed)};
-    if (publish_partials<1>(v, partials, &st->ticket[0])) {
-      const double a = sum_partials(ax_partials, ax_blocks, 1, 0, sRed);
-      const double b = sum_partials(partials, gridDim.x, 1, 0, sRed);
-      if (threadIdx.x == 0) {
-        const double pw = a + b;
-        st->pw = pw;
-        if (!(pw > 0.0) || !isfinite(pw)) {
-          st->status = SEM_ERR_BREAKDOWN;
-          st->done = 1;
-          st->alpha = 0.0;  // x is not advanced along this p (fused CG: nothing left to flush)
-        } else {
-          st->alpha = st->rho / pw;
-        }
-      }
-    }
   }
 }
 
@@ -207,24 +175,13 @@ sem_status launch_dssum(sem_prec prec, const GsPlan& g, void* u, int apply_mask,
   return SEM_OK;
 }
 
-sem_status launch_dssum_cg(sem_prec prec, const GsPlan& g, void* w, const void* p, CgScalars* st,
-                           const double* ax_partials, int ax_blocks, double* partials, cudaStream_t s) {
-  const int grid = seg_grid(g.total());
-  if (prec == SEM_F64) {
-    if (p)
-      k_dssum_cg<double, true><<<grid, kThreads, 0, s>>>(g, static_cast<double*>(w), static_cast<const double*>(p),
-                                                         st, ax_partials, ax_blocks, partials);
-    else
-      k_dssum_cg<double, false><<<grid, kThreads, 0, s>>>(g, static_cast<double*>(w), nullptr, st, ax_partials,
-                                                          ax_blocks, partials);
-  } else {
-    if (p)
-      k_dssum_cg<float, true><<<grid, kThreads, 0, s>>>(g, static_cast<float*>(w), static_cast<const float*>(p), st,
-                                                        ax_partials, ax_blocks, partials);
-    else
-      k_dssum_cg<float, false><<<grid, kThreads, 0, s>>>(g, static_cast<float*>(w), nullptr, st, ax_partials,
-                                                         ax_blocks, partials);
-  }
+sem_status launch_dssum_cg(sem_prec prec, const GsPlan& g, void* w, CgScalars* st, const double* ax_partials,
+                           int ax_blocks, cudaStream_t s) {
+  const int grid = seg_grid(g.total() + kThreads);  // block 0 and the segments'; at least two
+  if (prec == SEM_F64)
+    k_dssum_cg<double><<<grid, kThreads, 0, s>>>(g, static_cast<double*>(w), st, ax_partials, ax_blocks);
+  else
+    k_dssum_cg<float><<<grid, kThreads, 0, s>>>(g, static_cast<float*>(w), st, ax_partials, ax_blocks);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;

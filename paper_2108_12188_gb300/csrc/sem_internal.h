@@ -384,11 +384,7 @@ sem_status launch_cast(int64_t n, const double* in, float* out, cudaStream_t s);
 
 // gather-scatter (k_gs.cu)
 sem_status launch_dssum(sem_prec prec, const GsPlan& g, void* u, int apply_mask, cudaStream_t s);
-// CG variant: with p, also the boundary part of <p, w, c> (the operator added the interior
-// part), and the last block combines the partials and sets alpha (or a breakdown status);
-// with p == nullptr the operator's partials hold the whole product (whole_dot) and block 0
-// sums them and sets alpha before its share of the segments.
-inline bool whole_dot(sem_prec) { return true; }  // every CG-mode operator forms the whole <p, w>
+// CG variant: block 0 adds the operator's partials of <p, w, c> and sets alpha (or a breakdown status).
 // The CG layout (CgMap) is used for FP64 data (FP64 and double-float operators): their w does not
 // fit in L2 and the gather-scatter is bound by DRAM sectors. FP32 CG keeps the local layout (its
 // w stays in L2, and reading w through the map costs the FP32 update more than it saves).
@@ -399,8 +395,8 @@ inline bool cg_layout(sem_prec prec) { return prec != SEM_F32; }
 inline bool fused_cg(sem_prec prec, int N, sem_ax_variant v) {
   return prec != SEM_F64 || (v == SEM_AX_STORED && ax_slice_order(N));
 }
-sem_status launch_dssum_cg(sem_prec prec, const GsPlan& g, void* w, const void* p, CgScalars* st,
-                           const double* ax_partials, int ax_blocks, double* partials, cudaStream_t s);
+sem_status launch_dssum_cg(sem_prec prec, const GsPlan& g, void* w, CgScalars* st, const double* ax_partials,
+                           int ax_blocks, cudaStream_t s);
 // Batched kernels (k_batch.cu) over the device table `t` (host copy `h` gives the orders present
 // and is read on the host only). One CG iteration: an operator launch per order present, then
 // the gather-scatter and the update; the flush ends a run of iterations. launch_batch_status copies
