@@ -201,7 +201,7 @@ void resolve_variant(sem_mesh m, sem_prec prec, sem_ax_variant v, sem_ax_variant
     if (prec == SEM_F64X && r == SEM_AX_OTF_SCALE) r = has_factors(m, prec) ? SEM_AX_STORED : SEM_AX_OTF;
   }
   *out_v = r;
-  *out_shape = t.valid ? t.shape[vslot(r)] : 0;
+  *out_shape = t.valid ? t.shape[vslot(r)] : kUntunedShape;
 }
 
 }  // namespace

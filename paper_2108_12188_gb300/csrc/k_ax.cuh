@@ -608,16 +608,33 @@ inline int device_sm_count() {
   return n;
 }
 
+// The shape an untuned launch takes, from the tuner's times at 16.8M points (default / alternative):
+// FP32 on the fly N = 6 101.5 / 88.5, N = 7 77.2 / 67.7, N = 8 92.0 / 80.0 us (one or two elements per block
+// instead of two or three: more blocks to hide the barriers of each); FP64 N = 9 on the fly 4.07 /
+// 3.58, stored 2.27 / 2.03 ms (two elements of 100 threads fill 6.25 of 7 warps, one 3.1 of 4). Elsewhere
+// the default is the faster one or within 4%.
+template <int NP, typename T>
+constexpr bool ax_untuned_alt(sem_ax_variant v) {
+  return std::is_same_v<T, double> ? NP == 10 : v == SEM_AX_OTF && NP >= 7 && NP <= 9;
+}
+
 // A mesh with fewer element groups than SMs takes the shape with fewer elements per block
 // (if there is one), so that more SMs share its FP64 work.
 template <int NP, typename T>
 sem_status launch_ax_np(int N, sem_ax_variant v, bool cg, const AxLaunch& a, cudaStream_t s) {
   if (v == SEM_AX_OTF_SCALE)
     return cg ? launch_ax_t<NP, T, 2, true, ax_epb<NP>()>(N, a, s) : launch_ax_t<NP, T, 2, false, ax_epb<NP>()>(N, a, s);
-  const bool few_groups = a.shape == 0 && (a.E + ax_epb<NP>() - 1) / ax_epb<NP>() < device_sm_count();
-  if ((a.shape == 1 && ax_epb_alt<NP>() != ax_epb<NP>()) || (few_groups && ax_epb_alt<NP>() < ax_epb<NP>()))
-    return launch_ax_shape<NP, T, ax_epb_alt<NP>()>(N, v, cg, a, s);
-  return launch_ax_shape<NP, T, ax_epb<NP>()>(N, v, cg, a, s);
+  constexpr int kDef = ax_epb<NP>(), kAlt = ax_epb_alt<NP>();
+  bool alt = a.shape == 1 || (a.shape == kUntunedShape && ax_untuned_alt<NP, T>(v));
+  if (a.shape == 0 || a.shape == kUntunedShape) {
+    const int64_t groups = (a.E + (alt ? kAlt : kDef) - 1) / (alt ? kAlt : kDef);
+    if (groups < device_sm_count()) alt = kAlt < kDef;
+    // more elements per block than the default: not for the second wave of one and a bit (343 elements, FP64 on
+    // the fly at N = 9: 125 us in twos, 109 singly; 512 elements stored 74 and 82)
+    if (alt && kAlt > kDef && 2 * groups < 3 * device_sm_count()) alt = false;
+  }
+  if (alt && kAlt != kDef) return launch_ax_shape<NP, T, kAlt>(N, v, cg, a, s);
+  return launch_ax_shape<NP, T, kDef>(N, v, cg, a, s);
 }
 
 // Orders LO..HI (points per direction) of one precision; each translation unit compiles a range.
