@@ -54,7 +54,7 @@ typedef enum {
 } sem_status;
 
 /* SEM_F64: FP64 data and arithmetic of FP64 accuracy: FP64 instructions, and with SEM_AX_STORED at
- * orders 3, 5, 6 and 7 exact integer products on the tensor cores with 64-bit fixed point (elements
+ * orders 3, 5 to 7 and 9 to 11 exact integer products on the tensor cores with 64-bit fixed point (elements
  * that hold infinities, NaN or values near the ends of the FP64 range take FP64 instructions). SEM_F32: FP32 data and arithmetic.
  * SEM_F64X: FP64 data (double* vectors, FP64 stored factors); the local operator runs in
  * double-float arithmetic (pairs of floats with error-free products and sums, about 47
@@ -62,9 +62,9 @@ typedef enum {
  * sem_ax (and the CG options' f64_arith) use it: with SEM_AX_STORED on the float-pair factors of
  * SEM_MESH_F64X_STORED if the mesh has them, else the FP64 ones; with SEM_AX_OTF on factors
  * rebuilt from the element's trilinear coefficients (the per-column polynomial coefficients
- * in FP64, every point in double-float); SEM_AX_OTF_SCALE gives SEM_ERR_UNSUPPORTED. At order 7 SEM_AX_STORED is
- * the operator of SEM_F64, which is the faster one there. Every other call treats SEM_F64X like SEM_F64. Values below 2^-126 in magnitude are flushed to
- * zero inside it. */
+ * in FP64, every point in double-float); SEM_AX_OTF_SCALE gives SEM_ERR_UNSUPPORTED. At order 7
+ * SEM_AX_STORED is the operator of SEM_F64, which is the faster one there. Every other call treats
+ * SEM_F64X like SEM_F64. Values below 2^-126 in magnitude are flushed to zero inside it. */
 typedef enum { SEM_F64 = 0, SEM_F32 = 1, SEM_F64X = 2 } sem_prec;
 
 /* Variants of the local operator A_L (Section 5.1):
@@ -81,7 +81,7 @@ typedef enum { SEM_AX_STORED = 0, SEM_AX_OTF = 1, SEM_AX_AUTO = 2, SEM_AX_OTF_SC
 
 /* Flags for sem_mesh_create: which stored-factor arrays to keep on the device.
  * The per-element coefficients for the OTF variant are always kept (FP64 and FP32). */
-#define SEM_MESH_F64_STORED 1u /* G for SEM_F64: 48 bytes per local point (FP64; 64-bit fixed point at orders 3, 5, 6, 7) */
+#define SEM_MESH_F64_STORED 1u /* G for SEM_F64: 48 bytes per local point (FP64; 64-bit fixed point at orders 3, 5-7, 9-11) */
 #define SEM_MESH_F32_STORED 2u /* G in FP32: 24 bytes per local point */
 #define SEM_MESH_OTF_SCALE 4u  /* w_i w_j w_k / det J per point, FP64 and FP32: 12 bytes per local point */
 #define SEM_MESH_F64X_STORED 8u /* G as float pairs (high, low: 48 significant bits) for SEM_F64X: 48 bytes
@@ -313,7 +313,7 @@ sem_status sem_cg_solve(sem_mesh mesh, const double* b_dev, double* x_dev, const
  *  sem_cg_iterate  enqueues k iterations (a captured graph when opts.use_graph);
  *                  iterations after convergence are no-ops; async; when they have run,
  *                  x_dev holds the iterate of the last one (with opts.f64_arith, and with
- *                  stored factors at orders 3, 5, 6, 7, the operator makes each x update
+ *                  stored factors at orders 3, 5-7, 9-11, the operator makes each x update
  *                  one iteration late, and the call ends with the pending one);
  *  sem_cg_query    synchronises `stream` and reports iterations, residual, status;
  *  sem_cg_destroy  frees the handle. x_dev passed to sem_cg_start is updated in place

@@ -611,7 +611,7 @@ inline int device_sm_count() {
 // The shape an untuned launch takes, from the tuner's times at 16.8M points (default / alternative):
 // FP32 on the fly N = 6 101.5 / 88.5, N = 7 77.2 / 67.7, N = 8 92.0 / 80.0 us (one or two elements per block
 // instead of two or three: more blocks to hide the barriers of each); FP64 N = 9 on the fly 4.07 /
-// 3.58, stored 2.27 / 2.03 ms (two elements of 100 threads fill 6.25 of 7 warps, one 3.1 of 4). Elsewhere
+// 3.58 ms (two elements of 100 threads fill 6.25 of 7 warps, one 3.1 of 4). Elsewhere
 // the default is the faster one or within 4%.
 template <int NP, typename T>
 constexpr bool ax_untuned_alt(sem_ax_variant v) {
@@ -630,7 +630,7 @@ sem_status launch_ax_np(int N, sem_ax_variant v, bool cg, const AxLaunch& a, cud
     const int64_t groups = (a.E + (alt ? kAlt : kDef) - 1) / (alt ? kAlt : kDef);
     if (groups < device_sm_count()) alt = kAlt < kDef;
     // more elements per block than the default: not for the second wave of one and a bit (343 elements, FP64 on
-    // the fly at N = 9: 125 us in twos, 109 singly; 512 elements stored 74 and 82)
+    // the fly at N = 9: 125 us in twos, 109 singly)
     if (alt && kAlt > kDef && 2 * groups < 3 * device_sm_count()) alt = false;
   }
   if (alt && kAlt != kDef) return launch_ax_shape<NP, T, kAlt>(N, v, cg, a, s);

@@ -1,5 +1,5 @@
 // FP64 operator with stored factors on the tensor cores (k_ax_slice.cuh) at the orders of
-// ax_slice_order.
+// ax_slice_order, up to 8 points per direction.
 #include "k_ax_slice.cuh"
 
 namespace sem {
@@ -15,6 +15,8 @@ sem_status launch_slice(int N, bool cg, const AxLaunch& a, cudaStream_t s) {
 
 }  // namespace
 
-sem_status launch_ax_slice(int N, bool cg, const AxLaunch& a, cudaStream_t s) { return launch_slice<2>(N, cg, a, s); }
+sem_status launch_ax_slice(int N, bool cg, const AxLaunch& a, cudaStream_t s) {
+  return N <= 7 ? launch_slice<2>(N, cg, a, s) : launch_ax_slice_hi(N, cg, a, s);
+}
 
 }  // namespace sem

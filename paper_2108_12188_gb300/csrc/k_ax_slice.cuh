@@ -63,8 +63,10 @@ constexpr uint32_t kMagicBits = 0x4b400000u;
 // digit t (top digit first); M = digits * 2^-e. The rows of D (and with them the columns of D^T)
 // are scaled by 2^-fixed_row_scale. For NP <= 4 the matrix repeats along the diagonal, once per element
 // of the block's row of elements; entries beyond NP points are zero.
+template <int NP>
 struct SliceTab {
-  uint32_t d[2][kSlices][8][4];
+  static constexpr int R = NP <= 8 ? 8 : 16;
+  uint32_t d[2][kSlices][R][R / 2];
   int e;
 };
 
@@ -83,18 +85,23 @@ inline uint32_t half_bits(int v) {  // |v| <= 2048: exact
   return b;
 }
 
-// The largest e such that |D 2^e| <= 511 2^50, every |C_g| (g < 5) stays below 2^22 for any digits
-// |u_0| <= 256, |u_s| <= 512, and |V| = |U D 2^e| / 2^57 stays below 2^61.
+// Groups that accumulate on top of kMagic: as many as stay below 2^22 at the order without giving up more
+// than one bit of D (five groups would cost N = 9 four bits of D, four N = 11 four).
+__host__ __device__ constexpr int magic_groups(int NP) { return NP <= 8 ? 5 : NP <= 11 ? 4 : 3; }
+
+// The largest e such that |D 2^e| <= 511 2^50, every |C_g| that accumulates on kMagic stays below 2^22
+// for any digits |u_0| <= 256, |u_s| <= 512, and |V| = |U D 2^e| / 2^57 stays below 2^61.
 template <int NP>
-SliceTab make_slice_tab(int N) {
+SliceTab<NP> make_slice_tab(int N) {
+  constexpr int kGroups = magic_groups(NP), R = SliceTab<NP>::R;
   const GllTable& t = gll_table(N);
-  SliceTab r{};
+  SliceTab<NP> r{};
   for (int e = 60;; --e) {
     bool ok = true;
     int dig[2][kSlices][NP][NP];
     for (int m = 0; m < 2 && ok; ++m)
       for (int i = 0; i < NP && ok; ++i) {
-        double sum = 0.0, cg[5] = {0, 0, 0, 0, 0};
+        double sum = 0.0, cg[kGroups] = {};
         for (int l = 0; l < NP && ok; ++l) {
           const double v = std::ldexp(m == 0 ? t.D[i * NP + l] : t.D[l * NP + i], e - fixed_row_scale(NP, m == 0 ? i : l));
           ok = std::fabs(v) <= std::ldexp(511.0, 50);
@@ -107,7 +114,7 @@ SliceTab make_slice_tab(int N) {
             x = (x - low) >> 10;
           }
           dig[m][0][i][l] = static_cast<int>(x);
-          for (int g = 0; g < 5; ++g)
+          for (int g = 0; g < kGroups; ++g)
             for (int s = 0; s <= g; ++s) cg[g] += (s == 0 ? 256.0 : 512.0) * std::abs(dig[m][g - s][i][l]);
         }
         for (double c : cg) ok = ok && c < 4194304.0;
@@ -119,8 +126,8 @@ SliceTab make_slice_tab(int N) {
       for (int q = 0; q < kSlices; ++q)
         for (int i = 0; i < NP; ++i)
           for (int l = 0; l < NP; ++l)
-            for (int b = 0; b < 8; b += slice_width(NP))
-              r.d[m][q][b + i][(b + l) / 2] |= half_bits(dig[m][q][i][l]) << (16 * (l % 2));
+            for (int b = 0; b < (NP <= 8 ? 8 : 1); b += slice_width(NP))
+              r.d[m][q][(b + i) % R][(b + l) / 2 % (R / 2)] |= half_bits(dig[m][q][i][l]) << (16 * (l % 2));
     return r;
   }
 }
@@ -317,7 +324,7 @@ __device__ __forceinline__ double to_double(long long v, int k) {
 }
 
 // The element in FP64, as k_ax computes it (lines through the even/odd split of D): w of the whole
-// element to out[k * 72 + j * 8 + i]. scratch: 3 NP^3 doubles of shared memory. Called by all threads.
+// element to out[0 .. NP^3). scratch: 3 NP^3 doubles of shared memory. Called by all threads.
 template <int NP>
 __device__ __noinline__ void element_fp64(const GllParam<NP, double>& tab, const double* __restrict__ u,
                                           const int2* __restrict__ G, int sg, double* scratch, double* out) {
@@ -359,7 +366,7 @@ __device__ __noinline__ void element_fp64(const GllParam<NP, double>& tab, const
   lines(tab.Dt, A, A, 1, NP2, NP);
   lines(tab.Dt, C, C, 1, NP, NP2);
   __syncthreads();
-  for (int q = t; q < P; q += nt) out[(q / NP2) * 72 + (q / NP % NP) * 8 + q % NP] = B[q] + A[q] + C[q];
+  for (int q = t; q < P; q += nt) out[q] = B[q] + A[q] + C[q];
   __syncthreads();
 }
 
@@ -408,7 +415,7 @@ __device__ __forceinline__ unsigned over_element(unsigned v, F&& op) {
 // The factors of the next group arrive by one TMA bulk copy during phase 3 and the next phase 0.
 template <int NP, bool CG>
 __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
-    k_ax_slice(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab sl, int64_t E,
+    k_ax_slice(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab<NP> sl, int64_t E,
                const double* __restrict__ u, double* __restrict__ w, const int2* __restrict__ G,
                const int* __restrict__ gexp, const double* __restrict__ r, const double* __restrict__ minv,
                double* __restrict__ x, double* __restrict__ p, CgScalars* __restrict__ st,
@@ -754,17 +761,16 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
         wv[t][1] = to_double(sum[t][1] + r.y, scale);
       }
     } else {
+      double* scratch = reinterpret_cast<double*>(sG);  // the copy has landed; G is read from memory
+      double* res = scratch + 3 * P;
       for (int q = 0; q < S::kElems && e0 + q < E; ++q)
-        element_fp64<NP>(tab, (CG ? p : u) + (e0 + q) * P, G + (e0 + q) * 6 * P, __ldg(gexp + e0 + q),
-                         reinterpret_cast<double*>(sG),
-                         reinterpret_cast<double*>(sX) +
-                             S::kW * (q / (S::kSub * S::kSub) * PL + q / S::kSub % S::kSub * 8 + q % S::kSub));
-      if (threadIdx.x == 0 && more) load_factors(grp + gridDim.x);
+        element_fp64<NP>(tab, (CG ? p : u) + (e0 + q) * P, G + (e0 + q) * 6 * P, __ldg(gexp + e0 + q), scratch, res + q * P);
 #pragma unroll
       for (int t = 0; t < 2; ++t)
 #pragma unroll
-        for (int x = 0; x < 2; ++x)
-          wv[t][x] = in[t][x] ? reinterpret_cast<const double*>(sX)[(k0 + t) * PL + j * 8 + i0 + x] : 0.0;
+        for (int x = 0; x < 2; ++x) wv[t][x] = in[t][x] ? res[own * P + t * NP2 + off + x] : 0.0;
+      __syncthreads();
+      if (threadIdx.x == 0 && more) load_factors(grp + gridDim.x);
     }
     if constexpr (CG) {
 #pragma unroll
@@ -797,7 +803,7 @@ sem_status launch_slice_t(int N, const AxLaunch& a, cudaStream_t s) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ax_slice<NP, CG>, S::kThreads, S::kBytes);
     return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
   }();
-  static const SliceTab sl = make_slice_tab<NP>(N);
+  static const SliceTab<NP> sl = make_slice_tab<NP>(N);
   static const GllParam<NP, double> tab = make_gll_param<NP, double>(N);
   const int64_t groups = (a.E + S::kElems - 1) / S::kElems;
   int grid = max_blocks < kRedMax ? max_blocks : kRedMax;

@@ -394,8 +394,11 @@ sem_status launch_geometry(int N, int64_t E, const double* coef64, double* G64, 
 }
 
 sem_status launch_fixed_factors(int N, int64_t E, const double* coef64, int2* X, int* gexp, int* bad, cudaStream_t s) {
-  const int P = (N + 1) * (N + 1) * (N + 1);  // 24 KB of shared memory at N = 7, the largest ax_slice_order
-  k_fixed_factors<<<static_cast<unsigned>(E), P < 128 ? 64 : 128, 6 * static_cast<size_t>(P) * sizeof(double), s>>>(
+  const int P = (N + 1) * (N + 1) * (N + 1);
+  static const cudaError_t attr = cudaFuncSetAttribute(k_fixed_factors, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       6 * kMaxNp * kMaxNp * kMaxNp * static_cast<int>(sizeof(double)));
+  SEM_CUDA_TRY(attr);
+  k_fixed_factors<<<static_cast<unsigned>(E), P < 128 ? 64 : P < 600 ? 128 : 256, 6 * static_cast<size_t>(P) * sizeof(double), s>>>(
       gll_all(N), N + 1, coef64, X, gexp, bad);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());

@@ -133,15 +133,16 @@ inline int64_t factor_stride(int Np, bool fp32) {
   return fp32 ? (s + 3) / 4 * 4 : s;
 }
 
-// Orders whose FP64 stored-factor operator runs on the tensor cores (k_ax_slice.cuh). Their meshes
-// keep G as 64-bit fixed point instead of FP64, in the same bytes: X = G_ab 2^(sg + c_a + c_b), |X| <=
-// 2^59, as 32-bit signed halves (low, high), with sg per element and c = fixed_row_scale of the
+// Orders whose FP64 stored-factor operator runs on the tensor cores (k_ax_slice.cuh, k_ax_slice16.cuh).
+// Their meshes keep G as 64-bit fixed point instead of FP64, in the same bytes: X = G_ab 2^(sg + c_a + c_b),
+// |X| <= 2^59, as 32-bit signed halves (low, high), with sg per element and c = fixed_row_scale of the
 // point's index along each direction. At 16.8M points the FP64 kernel against this one: N = 3 1.12 and
-// 0.36 ms, N = 5 1.50 and 0.79, N = 6 1.52 and 0.62, N = 7 1.50 and 0.36. N = 2 and 4 fill too little of
-// the 8 x 8 x 8 points a block works on (0.86 against 0.93 ms, 1.13 against 1.31). At N = 1 the FP64
-// differences of equal values are exact zeros, which fixed-point factors do not keep on stretched
-// elements (relative error 1.4e-15 against 1.2e-16 at aspect ratio 100).
-__host__ __device__ constexpr bool ax_slice_order(int N) { return N == 3 || N == 5 || N == 6 || N == 7; }
+// 0.36 ms, N = 5 1.50 and 0.75, N = 6 1.52 and 0.59, N = 7 1.50 and 0.34, N = 9 2.03 and 1.51, N = 10 1.79 and
+// 1.08, N = 11 2.06 and 0.85. N = 2, 4 and 8 fill too little of the boxes of 8 or 16 points a side that the
+// tensor cores work on (N = 2 0.86 against 0.93 ms, N = 4 1.13 against 1.31; 729 of 2304 points at N = 8). At
+// N = 1 the FP64 differences of equal values are exact zeros, which fixed-point factors do not keep on
+// stretched elements (relative error 1.4e-15 against 1.2e-16 at aspect ratio 100).
+__host__ __device__ constexpr bool ax_slice_order(int N) { return N == 3 || (N >= 5 && N <= 7) || (N >= 9 && N <= 11); }
 // SEM_F64X with stored factors runs there too at N = 7: it is the faster of the two and the more accurate
 // (A_L 0.344 against 0.409 ms in double-float at 16.8M points, a CG iteration 0.578 against 0.643; N = 3 0.36
 // against 0.27, N = 5 0.79 against 0.38, N = 6 0.62 against 0.50).
@@ -317,6 +318,7 @@ sem_status launch_ax_f32_lo(int N, sem_ax_variant v, bool cg_mode, const AxLaunc
 sem_status launch_ax_f32_hi(int N, sem_ax_variant v, bool cg_mode, const AxLaunch& a, cudaStream_t s);
 // FP64 with stored (fixed-point) factors on the tensor cores, ax_slice_order only.
 sem_status launch_ax_slice(int N, bool cg_mode, const AxLaunch& a, cudaStream_t s);
+sem_status launch_ax_slice_hi(int N, bool cg_mode, const AxLaunch& a, cudaStream_t s);  // N + 1 >= 9
 inline sem_status launch_ax_f64(int N, sem_ax_variant v, bool cg, const AxLaunch& a, cudaStream_t s) {
   if (v == SEM_AX_STORED && ax_slice_order(N)) return launch_ax_slice(N, cg, a, s);
   return N + 1 <= 7 ? launch_ax_f64_lo(N, v, cg, a, s) : launch_ax_f64_hi(N, v, cg, a, s);

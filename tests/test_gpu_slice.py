@@ -1,4 +1,4 @@
-"""FP64 operator on the tensor cores (stored factors, orders 3, 5, 6 and 7): A_L against the oracle
+"""FP64 operator on the tensor cores (stored factors, orders 3, 5 to 7 and 9 to 11): A_L against the oracle
 where its integer digits, element scales and shared blocks can go wrong.
 
 Tolerance: the FP64 parity gate, 1e-12 relative 2-norm (per element for the scaled fields). The operator is
@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 # (elements, N): one element; a block of eight N = 3 elements with one left over; ragged boxes
 CASES = [((1, 1, 1), 3), ((3, 3, 1), 3), ((2, 2, 2), 3), ((5, 3, 2), 3), ((1, 1, 1), 5), ((3, 2, 2), 5),
-         ((2, 2, 1), 6), ((1, 1, 1), 7), ((3, 2, 2), 7)]
+         ((2, 2, 1), 6), ((1, 1, 1), 7), ((3, 2, 2), 7), ((2, 2, 1), 9), ((1, 1, 1), 10), ((2, 1, 2), 10),
+         ((1, 2, 2), 11)]
 IDS = [f"{d[0]}x{d[1]}x{d[2]}-N{N}" for d, N in CASES]
 
 
@@ -65,7 +66,7 @@ def test_operator(sem, dims, N):
     assert err.max() <= 1e-12
 
 
-@pytest.mark.parametrize("dims,N", [((3, 3, 1), 3), ((3, 2, 2), 7)], ids=["N3", "N7"])
+@pytest.mark.parametrize("dims,N", [((3, 3, 1), 3), ((3, 2, 2), 7), ((5, 1, 1), 10)], ids=["N3", "N7", "N10"])
 def test_non_finite_values_stay_in_their_element(sem, dims, N):
     m = BoxMesh(*dims, jitter=0.15, seed=N)
     prob = so.SemProblem(N, m.vert_xyz, m.elem_verts)
