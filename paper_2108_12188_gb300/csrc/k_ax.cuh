@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(NP * NP * EPB)
             dot.add(rU[k], acc);
           } else if (valid) {
             const df2 a = df_from_double(rU[k]), b = df_from_double(acc);
-            df_fma_acc(bdot, a.h, a.l, b.h, b.l);
+            df_fma_acc_full(bdot, a.h, a.l, b.h, b.l);
           }
         }
       } else {

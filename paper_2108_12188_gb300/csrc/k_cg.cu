@@ -285,14 +285,14 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 5 : 4) k_cg_update(
     // point, and with them alpha and beta (x after 10 iterations on 8^3 elements: 5.1e-14 off a long-double
     // computation with the cut-off, 3.9e-15 without, in the same time).
     df2* sC = reinterpret_cast<df2*>(sRed);
-    for (int m = threadIdx.x; m < 256; m += blockDim.x) sC[m] = m == 1 ? df2{1.f, 0.f} : df_split<true>(ctab[m]);
+    for (int m = threadIdx.x; m < 256; m += blockDim.x) sC[m] = m == 1 ? df2{1.f, 0.f} : df_from_double(ctab[m]);
     __syncthreads();
     df2 rz{0.f, 0.f}, rr{0.f, 0.f};
     sweep([&](T& xi, T pi, T& ri, T wi, T& zi, T mi, unsigned m) {
       if constexpr (!FUSED) xi += alpha * pi;
       ri = ri - alpha * wi;
       zi = minv ? mi * ri : ri;
-      const df2 r2 = df_split<true>(ri), z2 = df_split<true>(zi), c2 = sC[m];
+      const df2 r2 = df_from_double(ri), z2 = df_from_double(zi), c2 = sC[m];
       float ch, cl;
       df_prod(c2.h, c2.l, r2.h, r2.l, ch, cl);
       df_fma_acc_full(rz, ch, cl, z2.h, z2.l);

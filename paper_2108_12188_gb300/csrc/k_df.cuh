@@ -9,9 +9,8 @@
 // which keeps about 47 significant bits (relative error ~1e-14).
 //
 // Conversions from FP64 use integer operations only (no FP64 instruction): h takes the top
-// 24 significand bits, l the next 23, cut off (df_from_double) or rounded to nearest
-// (df_split<true>). Values outside FP32's normal exponent range are not
-// representable this way: magnitudes below 2^-126 become 0, above 2^128 become inf.
+// 24 significand bits, l the next 23 rounded to nearest. Values outside FP32's normal exponent
+// range are not representable this way: magnitudes below 2^-126 become 0, above 2^128 become inf.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -22,10 +21,9 @@ struct df2 {
   float h, l;
 };
 
-// ROUND: the low part to nearest. Cutting every term of a long sum off the same way (by 2^-48 of
-// it on average) shifts the whole sum by that much, while rounding errors cancel.
-template <bool ROUND>
-__device__ __forceinline__ df2 df_split(double x) {
+// The low part is rounded to nearest: cutting every term of a long sum off the same way (by 2^-48
+// of it on average) shifts the whole sum by that much, while rounding errors cancel.
+__device__ __forceinline__ df2 df_from_double(double x) {
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
   const unsigned hi32 = static_cast<unsigned>(b >> 32), lo32 = static_cast<unsigned>(b);
   const unsigned sign = hi32 & 0x80000000u;
@@ -37,7 +35,7 @@ __device__ __forceinline__ df2 df_split(double x) {
     r.h = __uint_as_float(sign | (static_cast<unsigned>(fe) << 23) | mh);
     // the remaining 29 significand bits are rem * 2^(E - 1075); keep their top 23 exactly:
     // q is the integer rem >> 6, built without a conversion instruction
-    const unsigned rem23 = ((lo32 & 0x1fffffffu) + (ROUND ? 32u : 0u)) >> 6;  // at most 2^23
+    const unsigned rem23 = ((lo32 & 0x1fffffffu) + 32u) >> 6;  // at most 2^23
     const float q = __fsub_rn(__uint_as_float(0x4b000000u + rem23), 8388608.0f);
     const int se = E - 1069 + 127;  // biased exponent of 2^(E - 1069)
     const float scale = se >= 1 ? __uint_as_float(static_cast<unsigned>(se) << 23) : 0.0f;
@@ -52,8 +50,6 @@ __device__ __forceinline__ df2 df_split(double x) {
   }
   return r;
 }
-
-__device__ __forceinline__ df2 df_from_double(double x) { return df_split<false>(x); }
 
 // Two-wide FP32 subtraction (sm_100 and later), a - b in each lane, rounded to nearest; the
 // CUDA headers provide the add, multiply and multiply-add forms only.
