@@ -357,19 +357,41 @@ __device__ __forceinline__ void prefetch_factors(double* sG, const double* G, in
   }
 }
 
+// Minimum blocks per SM, which set the registers a thread may take: a block has few warps and a
+// barrier after each phase, so two blocks an SM leave it waiting. Left alone (1; 0: the compiler's
+// default) the CG prologue takes up to 250 registers. CG iterations in us with that against the
+// values here: stored as FP64 or fixed point N = 3 347 / 327 (8.0M points), N = 4 446 / 417 (8.0M),
+// N = 5 497 / 413 (8.5M), N = 6 810 / 490 (8.4M), N = 8 848 / 619 (7.8M), N = 9 650 / 607 (8.0M; the
+// plain kernel 441 / 405, as pairs 407 / 347); more blocks than these spill (N = 6 559 with four,
+// N = 8 735 with three). N = 10 and the lowest orders gain nothing. On the fly at N = 7 four (128
+// registers) in CG mode (0.429 -> 0.414 ms at 16.8M points).
+template <int NP, bool CG, int GK>
+__host__ __device__ constexpr int df_min_blocks() {
+  if (GK == kGkOtf) return NP == 8 && CG ? 4 : 0;
+  if (!CG) return NP == 10 ? 3 : 1;
+  return NP == 4 || NP == 5 ? 5 : NP == 6 ? 4 : NP == 7 || NP == 10 ? 3 : NP == 9 ? 2 : 1;
+}
+
+// On the fly the registers for more blocks cost a few spills, 1 to 4% where all blocks of a launch are
+// resident anyway, so this shape (0: none) is taken only by launches that df_min_blocks' shape
+// would run in more than one wave. CG iteration and plain kernel in us, that shape / this one, at 8M
+// points: N = 2 784 / 750 and 503 / 476, N = 4 725 / 696 and 421 / 396, N = 8 817 / 766 and 433 / 420, N = 9
+// 892 / 782 and 518 / 476, N = 10 799 / 696 and 397 / 384, N = 11 1403 / 972 and 879 / 551.
+template <int NP, bool CG, int GK>
+__host__ __device__ constexpr int df_dense_blocks() {
+  if (GK != kGkOtf) return 0;
+  return NP == 3 ? 4 : NP == 5 ? 5 : NP == 9 ? 3 : NP == 10 ? 4 : NP == 11 ? (CG ? 3 : 4) : NP == 12 ? 2 : 0;
+}
+
 // Phases of a group, as in k_ax (barrier between phases; each thread owns one i-row, one
 // j-line and one k-column of its element in the in-place phases):
 //   0 column of u (or x += alpha p, p = M^-1 r + beta p) -> registers and A;  1 i-rows of A -> ur into B, column -> ut;
 //   2 j-lines of A -> us in place;  3 column: G (ur, us, ut);  4 D^T on rows, lines, column;
 //   5 column: w = sum of the three, converted to FP64 and stored.
 // GK: the factors (kGkF64 / kGkPairs: stored, staged by TMA; kGkOtf: rebuilt from coef).
-// Minimum blocks per SM: four at N = 7 in CG mode and for the stored plain kernel (128
-// registers; 0.429 -> 0.414 ms against a minimum of 1); on the fly otherwise the compiler's
-// default (0: 128 registers at N = 7, 0.748 -> 0.707 ms against a minimum of 1); stored
-// otherwise 1 (the default took fewer registers there but ran 4% slower at N = 7).
-template <int NP, bool CG, int GK>
-__global__ void __launch_bounds__(NP * NP * ax_epb<NP>(),
-                                  (NP == 8 && (CG || GK != kGkOtf)) ? 4 : GK == kGkOtf ? 0 : 1)
+// MINB: minimum blocks per SM (df_min_blocks, df_dense_blocks).
+template <int NP, bool CG, int GK, int MINB>
+__global__ void __launch_bounds__(NP * NP * ax_epb<NP>(), MINB)
     k_ax_df(const __grid_constant__ DfTab<NP> tab, int64_t E, const double* __restrict__ u, double* __restrict__ w,
             const double* __restrict__ G, const int* __restrict__ gexp, const double* __restrict__ coef,
             const double* __restrict__ r,
@@ -613,24 +635,34 @@ __global__ void __launch_bounds__(NP * NP * ax_epb<NP>(),
   }
 }
 
-template <int NP, bool CG, int GK>
-sem_status launch_df_t(int N, const AxLaunch& a, cudaStream_t s) {
-  constexpr int EPB = ax_epb<NP>();
+// Resident blocks of a shape on the GPU, its dynamic shared-memory limit raised first; once.
+template <int NP, bool CG, int GK, int MINB>
+int df_max_blocks() {
   constexpr size_t smem = df_smem_bytes<NP, GK>();
-  // resident blocks per SM x SMs, with the dynamic shared-memory limit raised first; once
   static const int max_blocks = [] {
-    cudaFuncSetAttribute(k_ax_df<NP, CG, GK>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const auto kernel = k_ax_df<NP, CG, GK, MINB>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ax_df<NP, CG, GK>, NP * NP * EPB, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NP * NP * ax_epb<NP>(), smem);
     return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
   }();
+  return max_blocks;
+}
+
+template <int NP, bool CG, int GK, int MINB = df_min_blocks<NP, CG, GK>()>
+sem_status launch_df_t(int N, const AxLaunch& a, cudaStream_t s) {
+  constexpr int EPB = ax_epb<NP>(), kDense = df_dense_blocks<NP, CG, GK>();
+  const int max_blocks = df_max_blocks<NP, CG, GK, MINB>();
   const int64_t groups = (a.E + EPB - 1) / EPB;
+  if constexpr (kDense != 0 && MINB != kDense) {
+    if (groups > max_blocks) return launch_df_t<NP, CG, GK, kDense>(N, a, s);
+  }
   int grid = max_blocks < kRedMax ? max_blocks : kRedMax;
   if (groups < grid) grid = static_cast<int>(groups);
   if (a.grid_out) *a.grid_out = grid;
-  k_ax_df<NP, CG, GK><<<grid, NP * NP * EPB, smem, s>>>(
+  k_ax_df<NP, CG, GK, MINB><<<grid, NP * NP * EPB, df_smem_bytes<NP, GK>(), s>>>(
       make_df_tab<NP>(N), a.E, static_cast<const double*>(a.u), static_cast<double*>(a.w),
       static_cast<const double*>(a.G), a.gexp, static_cast<const double*>(a.coef), static_cast<const double*>(a.r),
       static_cast<double*>(a.p), static_cast<const double*>(a.minv), static_cast<double*>(a.x), a.st, a.partials,
