@@ -53,9 +53,10 @@ typedef enum {
   SEM_ERR_UNSUPPORTED = 9    /* e.g. polynomial order outside [1, SEM_MAX_N] */
 } sem_status;
 
-/* SEM_F64: FP64 data and arithmetic of FP64 accuracy: FP64 instructions, and with SEM_AX_STORED at
- * orders 3, 5 to 7 and 9 to 11 exact integer products on the tensor cores with 64-bit fixed point (elements
- * that hold infinities, NaN or values near the ends of the FP64 range take FP64 instructions). SEM_F32: FP32 data and arithmetic.
+/* SEM_F64: FP64 data and arithmetic of FP64 accuracy: FP64 instructions, and for the operator at orders 3,
+ * 5 to 7 and 9 to 11 exact integer products on the tensor cores with 64-bit fixed point (elements
+ * that hold infinities, NaN or values near the ends of the FP64 range take FP64 instructions, and so do
+ * meshes with elements so distorted that fixed point would lose precision on the fly). SEM_F32: FP32 data and arithmetic.
  * SEM_F64X: FP64 data (double* vectors, FP64 stored factors); the local operator runs in
  * double-float arithmetic (pairs of floats with error-free products and sums, about 47
  * significant bits) on the FP32 pipes, which GB300 issues 64 times faster than FP64. Only
@@ -72,7 +73,8 @@ typedef enum { SEM_F64 = 0, SEM_F32 = 1, SEM_F64X = 2 } sem_prec;
  * OTF recomputes them per point from 21 per-element trilinear-map coefficients;
  * OTF_SCALE recomputes them too but reads one word per point, w_i w_j w_k / det J, so the
  *   per-point division is not repeated (the rematerialisation of Section 5.1 with an I/O
- *   cost of one word per point); needs SEM_MESH_OTF_SCALE;
+ *   cost of one word per point); needs SEM_MESH_OTF_SCALE (SEM_F64 on the tensor cores rebuilds the
+ *   word too, which is faster there than reading it);
  * AUTO uses the variant and block shape sem_autotune found fastest for this order and
  * precision (before tuning: STORED if the mesh holds the factors, else OTF). */
 typedef enum { SEM_AX_STORED = 0, SEM_AX_OTF = 1, SEM_AX_AUTO = 2, SEM_AX_OTF_SCALE = 3 } sem_ax_variant;

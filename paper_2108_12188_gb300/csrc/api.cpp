@@ -126,6 +126,7 @@ void free_mesh(sem_mesh m) {
   dfree(m->G64, h);
   dfree(m->GI, h);
   dfree(m->gexp, h);
+  dfree(m->geo, h);
   dfree(m->G32, h);
   dfree(m->Gx, h);
   dfree(m->scale64, h);
@@ -214,6 +215,7 @@ sem_status launch_ax_any(sem_mesh m, sem_prec prec, sem_ax_variant v, bool cg, A
   a.coef = fp64_data ? static_cast<const void*>(m->coef64) : static_cast<const void*>(m->coef32);
   a.G = stored_factors(m, prec, &a.g_pairs);
   a.gexp = m->gexp;
+  a.geo = m->geo;
   a.scale = fp64_data ? static_cast<const void*>(m->scale64) : static_cast<const void*>(m->scale32);
   if (v == SEM_AX_STORED && !a.G)
     return fail(SEM_ERR_ARG, "stored factors of this precision were not requested at mesh creation");
@@ -369,6 +371,7 @@ extern "C" sem_status sem_mesh_create(int N, int64_t nv, const double* vert_xyz,
       SEM_STEP(dmalloc(&m->GI, static_cast<size_t>(E * 6 * P), &acc, s));
       SEM_STEP(dmalloc(&m->gexp, static_cast<size_t>(E), &acc, s));
     }
+    if (ax_slice_order(N)) SEM_STEP(dmalloc(&m->geo, static_cast<size_t>(E), &acc, s));
     if ((flags & SEM_MESH_F64X_STORED) && !x_fixed)
       SEM_STEP(dmalloc(&m->Gx, static_cast<size_t>(2 * E * 6 * P), &acc, s));
     if (flags & SEM_MESH_F32_STORED)
@@ -418,13 +421,17 @@ extern "C" sem_status sem_mesh_create(int N, int64_t nv, const double* vert_xyz,
     SEM_CSTEP(cudaMemsetAsync(bad, 0, sizeof(int), s));
     SEM_STEP(launch_coefficients(E, Xd, m->coef64, m->coef32, s));
     // geometric factors (and the det J > 0 check at every GLL point)
-    if (m->GI) SEM_STEP(launch_fixed_factors(N, E, m->coef64, m->GI, m->gexp, bad, s));
-    if (!m->GI || m->G64 || m->G32 || m->Gx || m->scale64) SEM_STEP(launch_geometry(N, E, m->coef64, m->G64, m->G32, nullptr, nullptr, bad, factor_stride(m->Np, false),
-                             factor_stride(m->Np, true), s, m->scale64, m->scale32, m->Gx));
+    SEM_STEP(launch_geometry(N, E, m->coef64, m->G64, m->G32, nullptr, nullptr, bad, factor_stride(m->Np, false),
+                             factor_stride(m->Np, true), s, m->scale64, m->scale32, m->Gx, m->GI, m->gexp, m->geo));
     int bad_h = 0;
     SEM_CSTEP(cudaMemcpyAsync(&bad_h, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     SEM_CSTEP(cudaStreamSynchronize(s));
-    if (bad_h) return cleanup(fail(SEM_ERR_MESH, "det J <= 0 (inverted or degenerate element)"));
+    if (bad_h & 2) {  // elements too distorted for factors rebuilt in fixed point: k_ax rebuilds them in FP64
+      dfree(m->geo, s);
+      m->geo = nullptr;
+      acc -= static_cast<size_t>(E) * sizeof(GeoElement);
+    }
+    if (bad_h & 1) return cleanup(fail(SEM_ERR_MESH, "det J <= 0 (inverted or degenerate element)"));
   #undef SEM_STEP
   #undef SEM_CSTEP
     cleanup(SEM_OK);
@@ -723,7 +730,7 @@ struct sem_cg_s {
 namespace sem {
 namespace {
 
-bool cg_fused(sem_cg c) { return fused_cg(c->prec, c->m->N, c->variant); }
+bool cg_fused(sem_cg c) { return fused_cg(c->prec, c->m->N, c->variant, c->m->geo); }
 
 const void* minv_of(sem_cg c) {
   if (!c->precond) return nullptr;
@@ -1370,6 +1377,7 @@ extern "C" sem_status sem_autotune(sem_mesh m, sem_prec prec, int reps, sem_tune
         a.coef = prec == SEM_F32 ? static_cast<const void*>(m->coef32) : static_cast<const void*>(m->coef64);
         a.G = stored_factors(m, prec, &a.g_pairs);
         a.gexp = m->gexp;
+        a.geo = m->geo;
         a.scale = prec == SEM_F32 ? static_cast<const void*>(m->scale32) : static_cast<const void*>(m->scale64);
         auto launch = [&] {
           if (prec == SEM_F64X) return launch_ax_f64x(m->N, v, false, a, s);

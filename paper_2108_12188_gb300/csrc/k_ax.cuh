@@ -610,7 +610,7 @@ inline int device_sm_count() {
 
 // The shape an untuned launch takes, from the tuner's times at 16.8M points (default / alternative):
 // FP32 on the fly N = 6 101.5 / 88.5, N = 7 77.2 / 67.7, N = 8 92.0 / 80.0 us (one or two elements per block
-// instead of two or three: more blocks to hide the barriers of each); FP64 N = 9 on the fly 4.07 /
+// instead of two or three: more blocks to hide the barriers of each); FP64 N = 9 on the fly (meshes without geo) 4.07 /
 // 3.58 ms (two elements of 100 threads fill 6.25 of 7 warps, one 3.1 of 4). Elsewhere
 // the default is the faster one or within 4%.
 template <int NP, typename T>

@@ -8,7 +8,7 @@ namespace {
 template <int NP>
 sem_status launch_slice(int N, bool cg, const AxLaunch& a, cudaStream_t s) {
   if constexpr (ax_slice_order(NP - 1))
-    if (N + 1 == NP) return cg ? launch_slice_t<NP, true>(N, a, s) : launch_slice_t<NP, false>(N, a, s);
+    if (N + 1 == NP) return cg ? launch_slice_t<NP, true, false>(N, a, s) : launch_slice_t<NP, false, false>(N, a, s);
   if constexpr (NP < 8) return launch_slice<NP + 1>(N, cg, a, s);
   return fail(SEM_ERR_UNSUPPORTED, "polynomial order not compiled in");
 }

@@ -1,5 +1,5 @@
-// FP64 local operator w = A_L u = D^T G D u (Eq. 4, Section 3.1) with stored factors, its line
-// contractions on the tensor cores with more than FP64 accuracy: the products run exactly, on
+// FP64 local operator w = A_L u = D^T G D u (Eq. 4, Section 3.1) with stored factors or with factors
+// rebuilt on the fly (k_geo_fixed.cuh), its line contractions on the tensor cores with more than FP64 accuracy: the products run exactly, on
 // integer digits (the error-free splitting of Ozaki, Ogita, Oishi and Rump, "Error-free
 // transformations of matrix multiplication by using fast routines of matrix multiplication and
 // its applications", Numerical Algorithms 59, 2012), and everything between the input and
@@ -33,6 +33,14 @@
 // 0.344 ms. In CG mode with the fused prologue 0.414 ms; it takes 0.02 ms from the operator's earlier
 // unfused form (0.394) and saves 0.067 in the update kernel: one Jacobi-CG iteration 1.793 -> 0.578 ms.
 //
+// On the fly (Section 5.1's rematerialised factors) the same kernel fills its factor buffer from the element's
+// coefficients, with about 700 instructions per point on the same pipes, still far below the 45 FP64 instructions
+// of k_ax for it. A_L in ms, k_ax and this kernel, 16M points: N = 3 2.72 and 1.10, N = 5 3.07 and 1.60, N = 6 2.98 and
+// 1.45, N = 7 2.63 and 0.90, N = 9 3.62 and 2.09, N = 10 3.13 and 1.78, N = 11 3.49 and 1.50 (of these the factors take
+// 0.5 ms, the row tables 0.05 and at N = 3 0.2); with the per-point scale of SEM_AX_OTF_SCALE, which is not read
+// here, 2.31, 2.67, 2.58, 2.30, 3.18, 2.75 and 3.15 before. Error against FP64 torch as with k_ax (N = 9 1.2e-15 and
+// 1.3e-15, N = 7 9.0e-16 and 9.3e-16).
+//
 // Error against 64 bits (relative 2-norm of w, N = 7, jittered elements, CPU model of both
 // kernels against an 80-bit reference; k_ax in brackets): random u 8e-17 (1.8e-16), a sine over 8^3
 // elements 4e-16 (1.4e-14), one plus 1e-8 of a sine 5e-9 (1.2e-6), aspect ratio 100 4e-12 (5e-11),
@@ -50,6 +58,7 @@
 #include <cmath>
 
 #include "k_ax.cuh"
+#include "k_geo_fixed.cuh"
 #include "k_tma.cuh"
 
 namespace sem {
@@ -324,10 +333,11 @@ __device__ __forceinline__ double to_double(long long v, int k) {
 }
 
 // The element in FP64, as k_ax computes it (lines through the even/odd split of D): w of the whole
-// element to out[0 .. NP^3). scratch: 3 NP^3 doubles of shared memory. Called by all threads.
-template <int NP>
-__device__ __noinline__ void element_fp64(const GllParam<NP, double>& tab, const double* __restrict__ u,
-                                          const int2* __restrict__ G, int sg, double* scratch, double* out) {
+// element to out[0 .. NP^3). factors(q, g): the six factors of point q. scratch: 3 NP^3 doubles of shared
+// memory. Called by all threads.
+template <int NP, typename F>
+__device__ __noinline__ void element_fp64(const GllParam<NP, double>& tab, const double* __restrict__ u, const F& factors,
+                                          double* scratch, double* out) {
   constexpr int NP2 = NP * NP, P = NP2 * NP;
   double *A = scratch, *B = A + P, *C = B + P;
   const int t = threadIdx.x, nt = blockDim.x;
@@ -349,13 +359,7 @@ __device__ __noinline__ void element_fp64(const GllParam<NP, double>& tab, const
   __syncthreads();
   for (int q = t; q < P; q += nt) {
     double g[6];
-    const int c[3] = {fixed_row_scale(NP, q % NP), fixed_row_scale(NP, q / NP % NP), fixed_row_scale(NP, q / NP2)};
-    for (int m = 0; m < 6; ++m) {
-      const int ra = m < 3 ? 0 : m < 5 ? 1 : 2, rb = m < 3 ? m : m < 5 ? m - 2 : 2;
-      const int2 x = G[m * P + q];
-      const long long v = static_cast<long long>(x.y) * 4294967296ll + x.x;
-      g[m] = scalbn(static_cast<double>(v), -(sg + c[ra] + c[rb]));
-    }
+    factors(q, g);
     const double ur = B[q], us = A[q], ut = C[q];
     B[q] = g[0] * ur + g[1] * us + g[2] * ut;
     A[q] = g[1] * ur + g[3] * us + g[4] * ut;
@@ -368,6 +372,109 @@ __device__ __noinline__ void element_fp64(const GllParam<NP, double>& tab, const
   __syncthreads();
   for (int q = t; q < P; q += nt) out[q] = B[q] + A[q] + C[q];
   __syncthreads();
+}
+
+// Its factors: fixed point (the element's block of G), or from the element's coefficients.
+template <int NP>
+struct StoredFactors {
+  const int2* G;
+  int sg;
+  __device__ __forceinline__ void operator()(int q, double (&g)[6]) const {
+    constexpr int NP2 = NP * NP, P = NP2 * NP;
+    const int c[3] = {fixed_row_scale(NP, q % NP), fixed_row_scale(NP, q / NP % NP), fixed_row_scale(NP, q / NP2)};
+    for (int m = 0; m < 6; ++m) {
+      const int ra = m < 3 ? 0 : m < 5 ? 1 : 2, rb = m < 3 ? m : m < 5 ? m - 2 : 2;
+      const int2 x = G[m * P + q];
+      const long long v = static_cast<long long>(x.y) * 4294967296ll + x.x;
+      g[m] = scalbn(static_cast<double>(v), -(sg + c[ra] + c[rb]));
+    }
+  }
+};
+template <int NP>
+struct OtfFactors {
+  const GllParam<NP, double>& tab;
+  const double* coef;
+  __device__ __forceinline__ void operator()(int q, double (&g)[6]) const {
+    constexpr int NP2 = NP * NP;
+    const int i = q % NP, j = q / NP % NP, k = q / NP2;
+    OtfColumn<double> geo;
+    geo.init(coef, tab.xi[i], tab.xi[j]);
+    const double gam = tab.xi[k], sc = tab.w[i] * tab.w[j] * tab.w[k] / geo.det(gam);
+    for (int a = 0; a < 3; ++a) {
+      double v[3] = {a == 0 ? 1.0 : 0.0, a == 1 ? 1.0 : 0.0, a == 2 ? 1.0 : 0.0};
+      geo.apply(gam, sc, v[0], v[1], v[2]);
+      for (int b = a; b < 3; ++b) g[a == 0 ? b : a + b + 1] = v[b];
+    }
+  }
+};
+
+// On the fly: the row tables of one group's elements in shared memory, and the group's factors from
+// them (k_geo_fixed.cuh). THREADS threads take kParts parts of every k-column.
+template <int NP, int ELEMS, int THREADS>
+struct OtfGeometry {
+  static constexpr int NP2 = NP * NP, P = NP2 * NP;
+  static constexpr int kParts = THREADS / (ELEMS * NP2) > 1 ? THREADS / (ELEMS * NP2) : 1;
+  struct Tables {
+    GeoEntry e[ELEMS][3][NP][3];
+    GeoEntryT t[ELEMS][NP][3];
+    GeoNodes<NP> n;
+    int one;
+  };
+  static __device__ __forceinline__ int one_of(const Tables* s) {
+    int one;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(one) : "r"(smem_u32(&s->one)));
+    return one;
+  }
+  static __device__ __forceinline__ void nodes(Tables* s, const GeoNodes<NP>& n) {
+    if (threadIdx.x < NP) {
+      s->n.x[threadIdx.x] = n.x[threadIdx.x];
+      s->n.w[threadIdx.x] = n.w[threadIdx.x];
+    }
+    if (threadIdx.x == 0) s->one = 1;
+  }
+  static __device__ __forceinline__ void rows(Tables* s, const GeoElement* __restrict__ geo, int64_t e0, int count) {
+    const int one = one_of(s);
+    for (int q = threadIdx.x; q < 9 * NP * count; q += THREADS) {
+      const int el = q / (9 * NP), d = q / (3 * NP) % 3, i = q / 3 % NP, c = q % 3;
+      s->e[el][d][i][c] = geo_entry(geo[e0 + el], d, c, s->n.x[i], one, &s->t[el][i][c]);
+    }
+  }
+  static __device__ __forceinline__ void columns(const Tables* s, const GeoElement* __restrict__ geo, int64_t e0, int count,
+                                                 int2* sG) {
+    const int one = one_of(s);
+    for (int q = threadIdx.x; q < NP2 * kParts * count; q += THREADS) {
+      const int el = q / (NP2 * kParts), part = q / NP2 % kParts, col = q % NP2, i = col % NP, j = col / NP;
+      const GeoEntry *e_i = s->e[el][0][i], *e_j = s->e[el][1][j];
+      const int down = __ldg(&geo[e0 + el].down), lz = __ldg(&geo[e0 + el].lz);
+      const int up = __ldg(&geo[e0 + el].up) & 255, b = __ldg(&geo[e0 + el].up) >> 8;
+      GeoColumn c;
+      c.init(e_i, e_j, s->t[el][i], s->n.x[i], s->n.x[j], s->n.w[i], s->n.w[j], one);
+      const int ci = fixed_row_scale(NP, i), cj = fixed_row_scale(NP, j);
+      int2* out = sG + el * 6 * P + col;
+#pragma unroll 1
+      for (int k = part * NP / kParts; k < (part + 1) * NP / kParts; ++k) {
+        const int ck = fixed_row_scale(NP, k);
+        const int sh[6] = {b + cj + ck - ci, b + ck, b + cj, b + ci + ck - cj, b + ci, b + ci + cj - ck};
+        c.point(e_i, e_j, s->e[el][2][k], s->n.x[k], s->n.w[k], down, lz, up, [&](int m, long long v) {
+          const Fx x = fx_split(v >> sh[m]);
+          out[m * P + k * NP2] = make_int2(x.l, x.h);
+        });
+      }
+    }
+  }
+};
+template <int NP>
+GeoNodes<NP> make_geo_nodes(int N) {
+  const GllTable& t = gll_table(N);
+  int c[NP];
+  for (int i = 0; i < NP; ++i) c[i] = fixed_row_scale(NP, i);
+  const int sw = geo_weight_scale(t.w, c, NP);
+  GeoNodes<NP> n{};
+  for (int i = 0; i < NP; ++i) {
+    n.x[i] = fx_split(std::llrint(std::ldexp(t.xi[i], 62)));
+    n.w[i] = fx_split(std::llrint(std::ldexp(t.w[i], 62 + sw + c[i])));
+  }
+  return n;
 }
 
 template <int NP>
@@ -390,7 +497,9 @@ struct SliceShape {
   static constexpr size_t kOffC = kOffB + 2 * 7 * 32 * 8;          // Start
   static constexpr size_t kOffM = kOffC + 32;                      // maxima [3][kElems][kSlots]
   static constexpr size_t kOffBar = kOffM + (3 * kElems * kSlots * 4 + 7) / 8 * 8;
-  static constexpr size_t kBytes = kOffBar + 8;
+  static constexpr size_t kOffTab = (kOffBar + 8 + 15) / 16 * 16;  // on the fly: row tables
+  using Geometry = OtfGeometry<NP, kElems, kThreads>;
+  static constexpr size_t bytes(bool otf) { return otf ? kOffTab + sizeof(typename Geometry::Tables) : kOffBar + 8; }
 };
 
 // OR or maximum of v over the lanes of the warp that hold points of one of the eight elements of a
@@ -413,11 +522,15 @@ __device__ __forceinline__ unsigned over_element(unsigned v, F&& op) {
 //   3  digits of vr and vs in registers (vs transposed), D^T on i-rows and j-lines, then (after a
 //      barrier) on k-lines, exchanged back; w
 // The factors of the next group arrive by one TMA bulk copy during phase 3 and the next phase 0.
-template <int NP, bool CG>
-__global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
-    k_ax_slice(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab<NP> sl, int64_t E,
-               const double* __restrict__ u, double* __restrict__ w, const int2* __restrict__ G,
-               const int* __restrict__ gexp, const double* __restrict__ r, const double* __restrict__ minv,
+// OTF: the factors are rebuilt (OtfGeometry: row tables in phase 0, the factors before phase 1) instead of
+// copied; three blocks per SM there (168 registers; N = 7 0.91 ms with four, 0.90 with three, N = 3 100 and 96 us at
+// 1.3M points), four at N = 5, whose blocks of 96 threads have the registers (CG 2.19 ms with three, 2.13 with four).
+template <int NP, bool CG, bool OTF>
+__global__ void __launch_bounds__(SliceShape<NP>::kThreads, OTF && NP != 6 ? 3 : 4)
+    k_ax_slice(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab<NP> sl,
+               const __grid_constant__ GeoNodes<NP> nodes, int64_t E, const double* __restrict__ u,
+               double* __restrict__ w, const int2* __restrict__ G, const int* __restrict__ gexp,
+               const double* __restrict__ coef, const GeoElement* __restrict__ geo, const double* __restrict__ r, const double* __restrict__ minv,
                double* __restrict__ x, double* __restrict__ p, CgScalars* __restrict__ st,
                double* __restrict__ partials, int* __restrict__ err) {
   using S = SliceShape<NP>;
@@ -458,7 +571,10 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
     mbar_expect_tx(bar, bytes);
     tma_load_1d(sG, G + grp * S::kElems * 6 * P, bytes, bar);
   };
-  if (threadIdx.x == 0) {
+  typename S::Geometry::Tables* tables = reinterpret_cast<typename S::Geometry::Tables*>(smem + S::kOffTab);
+  if constexpr (OTF) {
+    S::Geometry::nodes(tables, nodes);
+  } else if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     load_factors(blockIdx.x);
   }
@@ -557,7 +673,8 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
 #pragma unroll
       for (int t = 0; t < 2; ++t) load2(u, t, v[t]);
     }
-    const int sg = S::kElems == 1 || e < E ? __ldg(gexp + e) : 0;
+    if constexpr (OTF) S::Geometry::rows(tables, geo, e0, group_size(grp));
+    const int sg = S::kElems == 1 || e < E ? __ldg(OTF ? &geo[e].sg : gexp + e) : 0;
     unsigned mh = 0;
 #pragma unroll
     for (int t = 0; t < 2; ++t)
@@ -579,6 +696,9 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
       emax = 1080;
     }
     if (threadIdx.x == 0 && more) {  // the next group's vectors into L2
+      if constexpr (OTF)
+        l2_prefetch(geo + e0 + static_cast<int64_t>(gridDim.x) * S::kElems,
+                    static_cast<unsigned>(sizeof(GeoElement)) * group_size(grp + gridDim.x));
       if constexpr (P % 2 == 0) {
         const int64_t at = (e0 + static_cast<int64_t>(gridDim.x) * S::kElems) * P;
         const unsigned bytes = 8u * P * group_size(grp + gridDim.x);
@@ -601,6 +721,7 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
         for (int s = 0; s < kSlices; ++s) sD[(s * S::kDigit + (k0 + t) * PL) / 2 + lane] = d[s];
       }
     }
+    if constexpr (OTF) S::Geometry::columns(tables, geo, e0, group_size(grp), sG);
     const bool slow = __syncthreads_or(general);  // for the whole group
 
     // phase 1
@@ -650,7 +771,8 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
         m = over_element(m, by_or);
       put(1, own, m);
     }
-    const bool ok = mbar_wait_bounded(bar, parity);  // this group's factors
+    bool ok = true;
+    if constexpr (!OTF) ok = mbar_wait_bounded(bar, parity);  // this group's factors
     parity ^= 1u;
     if (__syncthreads_or(!ok)) {  // the factor copy did not arrive: report and leave together
       if (threadIdx.x == 0) {
@@ -739,7 +861,7 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
         sum[t][1] += r[1];
       }
       __syncthreads();  // the digits of vt; the factors are consumed
-      if (threadIdx.x == 0 && more) load_factors(grp + gridDim.x);
+      if (!OTF && threadIdx.x == 0 && more) load_factors(grp + gridDim.x);
       {
         uint32_t b[2][kSlices];
 #pragma unroll
@@ -763,14 +885,19 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
     } else {
       double* scratch = reinterpret_cast<double*>(sG);  // the copy has landed; G is read from memory
       double* res = scratch + 3 * P;
-      for (int q = 0; q < S::kElems && e0 + q < E; ++q)
-        element_fp64<NP>(tab, (CG ? p : u) + (e0 + q) * P, G + (e0 + q) * 6 * P, __ldg(gexp + e0 + q), scratch, res + q * P);
+      for (int q = 0; q < S::kElems && e0 + q < E; ++q) {
+        const double* src = (CG ? p : u) + (e0 + q) * P;
+        if constexpr (OTF)
+          element_fp64<NP>(tab, src, OtfFactors<NP>{tab, coef + (e0 + q) * 24}, scratch, res + q * P);
+        else
+          element_fp64<NP>(tab, src, StoredFactors<NP>{G + (e0 + q) * 6 * P, __ldg(gexp + e0 + q)}, scratch, res + q * P);
+      }
 #pragma unroll
       for (int t = 0; t < 2; ++t)
 #pragma unroll
         for (int x = 0; x < 2; ++x) wv[t][x] = in[t][x] ? res[own * P + t * NP2 + off + x] : 0.0;
       __syncthreads();
-      if (threadIdx.x == 0 && more) load_factors(grp + gridDim.x);
+      if (!OTF && threadIdx.x == 0 && more) load_factors(grp + gridDim.x);
     }
     if constexpr (CG) {
 #pragma unroll
@@ -792,26 +919,27 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, 4)
   }
 }
 
-template <int NP, bool CG>
+template <int NP, bool CG, bool OTF>
 sem_status launch_slice_t(int N, const AxLaunch& a, cudaStream_t s) {
   using S = SliceShape<NP>;
   static const int max_blocks = [] {
-    cudaFuncSetAttribute(k_ax_slice<NP, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(S::kBytes));
+    cudaFuncSetAttribute(k_ax_slice<NP, CG, OTF>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(S::bytes(OTF)));
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ax_slice<NP, CG>, S::kThreads, S::kBytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ax_slice<NP, CG, OTF>, S::kThreads, S::bytes(OTF));
     return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
   }();
   static const SliceTab<NP> sl = make_slice_tab<NP>(N);
   static const GllParam<NP, double> tab = make_gll_param<NP, double>(N);
+  static const GeoNodes<NP> nodes = make_geo_nodes<NP>(N);
   const int64_t groups = (a.E + S::kElems - 1) / S::kElems;
   int grid = max_blocks < kRedMax ? max_blocks : kRedMax;
   if (groups < grid) grid = static_cast<int>(groups);
   if (a.grid_out) *a.grid_out = grid;
-  k_ax_slice<NP, CG><<<grid, S::kThreads, S::kBytes, s>>>(
-      tab, sl, a.E, static_cast<const double*>(a.u), static_cast<double*>(a.w), static_cast<const int2*>(a.G), a.gexp,
-      static_cast<const double*>(a.r), static_cast<const double*>(a.minv), static_cast<double*>(a.x),
+  k_ax_slice<NP, CG, OTF><<<grid, S::kThreads, S::bytes(OTF), s>>>(
+      tab, sl, nodes, a.E, static_cast<const double*>(a.u), static_cast<double*>(a.w), static_cast<const int2*>(a.G),
+      a.gexp, static_cast<const double*>(a.coef), a.geo, static_cast<const double*>(a.r), static_cast<const double*>(a.minv), static_cast<double*>(a.x),
       static_cast<double*>(a.p), a.st, a.partials, a.err);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());

@@ -27,7 +27,9 @@ struct Slice16Shape {
   static constexpr size_t kOffT = kOffX + 2 * NP * kPlaneX * 8;   // fragments [2][kSlices][32] 16 bytes
   static constexpr size_t kOffM = kOffT + 2 * kSlices * 32 * 16;  // maxima [2][NP]
   static constexpr size_t kOffBar = kOffM + (2 * NP * 4 + 7) / 8 * 8;
-  static constexpr size_t kBytes = kOffBar + 8;
+  static constexpr size_t kOffTab = (kOffBar + 8 + 15) / 16 * 16;  // on the fly: row tables
+  using Geometry = OtfGeometry<NP, 1, kThreads>;
+  static constexpr size_t bytes(bool otf) { return otf ? kOffTab + sizeof(typename Geometry::Tables) : kOffBar + 8; }
 };
 
 // As combine() with fewer groups on top of kMagic: C_4 = 1024 t + r with t joining C_3, and for three groups
@@ -108,11 +110,12 @@ __device__ __forceinline__ long long value16(const float (&c)[7][4], int row, in
 // Warp k holds plane k; the lane's points are j = lane / 4 + 8 a, i = 2 (lane % 4) + 8 b + x (a, b, x in
 // {0, 1}), values [a][b][x]. Phases as in k_ax_slice; in the k contractions warp k takes the lines of plane
 // j = k.
-template <int NP, bool CG>
+template <int NP, bool CG, bool OTF>
 __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
-    k_ax_slice16(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab<NP> sl, int64_t E,
-                 const double* __restrict__ u, double* __restrict__ w, const int2* __restrict__ G,
-                 const int* __restrict__ gexp, const double* __restrict__ r, const double* __restrict__ minv,
+    k_ax_slice16(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab<NP> sl,
+                 const __grid_constant__ GeoNodes<NP> nodes, int64_t E, const double* __restrict__ u,
+                 double* __restrict__ w, const int2* __restrict__ G, const int* __restrict__ gexp,
+                 const double* __restrict__ coef, const GeoElement* __restrict__ geo, const double* __restrict__ r, const double* __restrict__ minv,
                  double* __restrict__ x, double* __restrict__ p, CgScalars* __restrict__ st,
                  double* __restrict__ partials, int* __restrict__ err) {
   using S = Slice16Shape<NP>;
@@ -139,7 +142,10 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
     mbar_expect_tx(bar, S::kElemBytes);
     tma_load_1d(sG, G + e * 6 * P, S::kElemBytes, bar);
   };
-  if (threadIdx.x == 0) {
+  typename S::Geometry::Tables* tables = reinterpret_cast<typename S::Geometry::Tables*>(smem + S::kOffTab);
+  if constexpr (OTF) {
+    S::Geometry::nodes(tables, nodes);
+  } else if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     load_factors(blockIdx.x);
   }
@@ -248,7 +254,8 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
           load2(u, a, b, v[a][b]);
         }
       }
-    const int sg = __ldg(gexp + e);
+    if constexpr (OTF) S::Geometry::rows(tables, geo, e, 1);
+    const int sg = __ldg(OTF ? &geo[e].sg : gexp + e);
     unsigned mh = 0;
     bool nonzero = false;
 #pragma unroll
@@ -273,6 +280,7 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
       emax = 1080;
     }
     if (threadIdx.x == 0 && more) {  // the next element's vectors into L2
+      if constexpr (OTF) l2_prefetch(geo + e + gridDim.x, sizeof(GeoElement));
       if constexpr (P % 2 == 0) {
         const int64_t at = (e + gridDim.x) * P;
         if constexpr (CG) {
@@ -293,6 +301,7 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
         digit_pairs(to_fixed(v[a][b][0], emax), to_fixed(v[a][b][1], emax), d);
         put_digits(a, b, d);
       }
+    if constexpr (OTF) S::Geometry::columns(tables, geo, e, 1, sG);
     const bool slow = __syncthreads_or(general);
 
     // phase 1
@@ -339,7 +348,8 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
       m = __reduce_or_sync(0xffffffffu, m);
       if (lane == 0) sMax[NP + warp] = m;
     }
-    const bool ok = mbar_wait_bounded(bar, parity);  // this element's factors
+    bool ok = true;
+    if constexpr (!OTF) ok = mbar_wait_bounded(bar, parity);  // this element's factors
     parity ^= 1u;
     if (__syncthreads_or(!ok)) {  // the factor copy did not arrive: report and leave together
       if (threadIdx.x == 0) {
@@ -439,7 +449,7 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
           for (int y = 0; y < 2; ++y) sum[a][b][y] += value16<kMg>(c, a, y);
       }
       __syncthreads();  // the digits of vt; the factors are consumed
-      if (threadIdx.x == 0 && more) load_factors(e + gridDim.x);
+      if (!OTF && threadIdx.x == 0 && more) load_factors(e + gridDim.x);
       k_lines(tT);
       __syncthreads();
       // w = sum 2^-sc: u 2^(1080 - emax), D 2^e / 2^57 twice, V 2^lv, G 2^sg / 2^64
@@ -455,7 +465,10 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
     } else {
       double* scratch = reinterpret_cast<double*>(sG);  // the copy has landed; G is read from memory
       double* res = scratch + 3 * P;
-      element_fp64<NP>(tab, (CG ? p : u) + e * P, G + e * 6 * P, sg, scratch, res);
+      if constexpr (OTF)
+        element_fp64<NP>(tab, (CG ? p : u) + e * P, OtfFactors<NP>{tab, coef + e * 24}, scratch, res);
+      else
+        element_fp64<NP>(tab, (CG ? p : u) + e * P, StoredFactors<NP>{G + e * 6 * P, sg}, scratch, res);
 #pragma unroll
       for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -463,7 +476,7 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
 #pragma unroll
           for (int y = 0; y < 2; ++y) wv[a][b][y] = in(a, b, y) ? res[warp * NP2 + off(a, b) + y] : 0.0;
       __syncthreads();
-      if (threadIdx.x == 0 && more) load_factors(e + gridDim.x);
+      if (!OTF && threadIdx.x == 0 && more) load_factors(e + gridDim.x);
     }
 #pragma unroll
     for (int a = 0; a < 2; ++a)
@@ -487,25 +500,26 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
   }
 }
 
-template <int NP, bool CG>
+template <int NP, bool CG, bool OTF>
 sem_status launch_slice16_t(int N, const AxLaunch& a, cudaStream_t s) {
   using S = Slice16Shape<NP>;
   static const int max_blocks = [] {
-    cudaFuncSetAttribute(k_ax_slice16<NP, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(S::kBytes));
+    cudaFuncSetAttribute(k_ax_slice16<NP, CG, OTF>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(S::bytes(OTF)));
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ax_slice16<NP, CG>, S::kThreads, S::kBytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ax_slice16<NP, CG, OTF>, S::kThreads, S::bytes(OTF));
     return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
   }();
   static const SliceTab<NP> sl = make_slice_tab<NP>(N);
   static const GllParam<NP, double> tab = make_gll_param<NP, double>(N);
+  static const GeoNodes<NP> nodes = make_geo_nodes<NP>(N);
   int grid = max_blocks < kRedMax ? max_blocks : kRedMax;
   if (a.E < grid) grid = static_cast<int>(a.E);
   if (a.grid_out) *a.grid_out = grid;
-  k_ax_slice16<NP, CG><<<grid, S::kThreads, S::kBytes, s>>>(
-      tab, sl, a.E, static_cast<const double*>(a.u), static_cast<double*>(a.w), static_cast<const int2*>(a.G), a.gexp,
-      static_cast<const double*>(a.r), static_cast<const double*>(a.minv), static_cast<double*>(a.x),
+  k_ax_slice16<NP, CG, OTF><<<grid, S::kThreads, S::bytes(OTF), s>>>(
+      tab, sl, nodes, a.E, static_cast<const double*>(a.u), static_cast<double*>(a.w), static_cast<const int2*>(a.G),
+      a.gexp, static_cast<const double*>(a.coef), a.geo, static_cast<const double*>(a.r), static_cast<const double*>(a.minv), static_cast<double*>(a.x),
       static_cast<double*>(a.p), a.st, a.partials, a.err);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());

@@ -8,7 +8,7 @@ namespace {
 template <int NP>
 sem_status launch_slice16(int N, bool cg, const AxLaunch& a, cudaStream_t s) {
   if constexpr (ax_slice_order(NP - 1))
-    if (N + 1 == NP) return cg ? launch_slice16_t<NP, true>(N, a, s) : launch_slice16_t<NP, false>(N, a, s);
+    if (N + 1 == NP) return cg ? launch_slice16_t<NP, true, false>(N, a, s) : launch_slice16_t<NP, false, false>(N, a, s);
   if constexpr (NP < 12) return launch_slice16<NP + 1>(N, cg, a, s);
   return fail(SEM_ERR_UNSUPPORTED, "polynomial order not compiled in");
 }

@@ -76,90 +76,169 @@ __device__ __forceinline__ void cross3(const double a[3], const double b[3], dou
   out[2] = a[0] * b[1] - a[1] * b[0];
 }
 
-// G = w |det J| J^-1 J^-T = (w / det) C C^T with C's rows c_b = g_{b+1} x g_{b+2}; B = w det.
-__device__ void point_geometry(const double* a, double xi, double eta, double gam, double wq, double G[6],
-                               double* B, double* det_out) {
+// C C^T with the cofactor rows c_b = g_{b+1} x g_{b+2}, and det J.
+__device__ void point_cofactors(const double* a, double xi, double eta, double gam, double cc[6], double* det_out) {
   double g0[3], g1[3], g2[3], c0[3], c1[3], c2[3];
   jacobian_columns(a, xi, eta, gam, g0, g1, g2);
   cross3(g1, g2, c0);
   cross3(g2, g0, c1);
   cross3(g0, g1, c2);
-  const double det = g0[0] * c0[0] + g0[1] * c0[1] + g0[2] * c0[2];
-  const double s = wq / det;
+  *det_out = g0[0] * c0[0] + g0[1] * c0[1] + g0[2] * c0[2];
   auto d = [](const double* p, const double* q) { return p[0] * q[0] + p[1] * q[1] + p[2] * q[2]; };
-  G[0] = s * d(c0, c0);
-  G[1] = s * d(c0, c1);
-  G[2] = s * d(c0, c2);
-  G[3] = s * d(c1, c1);
-  G[4] = s * d(c1, c2);
-  G[5] = s * d(c2, c2);
+  cc[0] = d(c0, c0);
+  cc[1] = d(c0, c1);
+  cc[2] = d(c0, c2);
+  cc[3] = d(c1, c1);
+  cc[4] = d(c1, c2);
+  cc[5] = d(c2, c2);
+}
+
+// G = w |det J| J^-1 J^-T = (w / det) C C^T; B = w det.
+__device__ void point_geometry(const double* a, double xi, double eta, double gam, double wq, double G[6],
+                               double* B, double* det_out) {
+  double det;
+  point_cofactors(a, xi, eta, gam, G, &det);
+  const double s = wq / det;
+  for (int m = 0; m < 6; ++m) G[m] = s * G[m];
   *B = wq * det;
   *det_out = det;
 }
 
+// Arrays of a mesh's geometry, each may be null: G in FP64, FP32 and as float pairs (high, low), B, and the scale of the
+// on-the-fly factors w / det J. gs64, gs32: words per element of G.
+struct GeometryOut {
+  double* G64;
+  float* G32;
+  double* B64;
+  float* B32;
+  int64_t gs64, gs32;
+  double* S64;
+  float* S32;
+  float* GX;
+  __device__ __forceinline__ void put(int64_t e, int P, int r, const double (&G)[6], double B, double sc) const {
+    for (int m = 0; m < 6; ++m) {
+      if (G64) G64[e * gs64 + m * P + r] = G[m];
+      if (G32) G32[e * gs32 + m * P + r] = static_cast<float>(G[m]);
+      if (GX) {  // high = G rounded to FP32, low = the rest rounded to FP32
+        const float h = static_cast<float>(G[m]);
+        GX[2 * (e * gs64 + m * P + r)] = h;
+        GX[2 * (e * gs64 + m * P + r) + 1] = static_cast<float>(G[m] - static_cast<double>(h));
+      }
+    }
+    const int64_t idx = e * P + r;
+    if (B64) B64[idx] = B;
+    if (B32) B32[idx] = static_cast<float>(B);
+    if (S64) S64[idx] = sc;
+    if (S32) S32[idx] = static_cast<float>(sc);
+  }
+};
+
 __global__ void k_geometry(const __grid_constant__ GllAll tab, int Np, int64_t E, const double* __restrict__ coef,
-                           double* __restrict__ G64, float* __restrict__ G32, double* __restrict__ B64,
-                           float* __restrict__ B32, int* __restrict__ bad, int64_t gs64, int64_t gs32,
-                           double* __restrict__ S64, float* __restrict__ S32, float* __restrict__ GX) {
+                           const __grid_constant__ GeometryOut out, int* __restrict__ bad) {
   const int64_t P = static_cast<int64_t>(Np) * Np * Np;
   const int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (idx >= E * P) return;
   const int64_t e = idx / P;
   const int r = static_cast<int>(idx - e * P);
   const int i = r % Np, j = (r / Np) % Np, k = r / (Np * Np);
+  const double wq = tab.w[i] * tab.w[j] * tab.w[k];
   double G[6], B, det;
-  point_geometry(coef + e * 24, tab.xi[i], tab.xi[j], tab.xi[k], tab.w[i] * tab.w[j] * tab.w[k], G, &B, &det);
+  point_geometry(coef + e * 24, tab.xi[i], tab.xi[j], tab.xi[k], wq, G, &B, &det);
   if (!(det > 0.0) || !isfinite(det)) atomicOr(bad, 1);
-  for (int m = 0; m < 6; ++m) {
-    if (G64) G64[e * gs64 + m * P + r] = G[m];
-    if (G32) G32[e * gs32 + m * P + r] = static_cast<float>(G[m]);
-    if (GX) {  // float pair (high, low): high = G rounded to FP32, low = the rest rounded to FP32
-      const float h = static_cast<float>(G[m]);
-      GX[2 * (e * gs64 + m * P + r)] = h;
-      GX[2 * (e * gs64 + m * P + r) + 1] = static_cast<float>(G[m] - static_cast<double>(h));
-    }
-  }
-  if (B64) B64[idx] = B;
-  if (B32) B32[idx] = static_cast<float>(B);
-  const double sc = tab.w[i] * tab.w[j] * tab.w[k] / det;  // scale of the on-the-fly factors
-  if (S64) S64[idx] = sc;
-  if (S32) S32[idx] = static_cast<float>(sc);
+  out.put(e, static_cast<int>(P), r, G, B, wq / det);
 }
 
-// G of one element per block as the fixed point of ax_slice_order: sg = 59 - (exponent of the
-// element's largest entry, row scales included). sG: 6 P doubles of dynamic shared memory.
-__global__ void k_fixed_factors(const __grid_constant__ GllAll tab, int Np, const double* __restrict__ coef,
-                                int2* __restrict__ X, int* __restrict__ gexp, int* __restrict__ bad) {
+// The same with one element per block at the orders of ax_slice_order, with G as their fixed point too: sg = 59 -
+// (exponent of the element's largest entry, row scales included), and the element for factors rebuilt on the fly (sw:
+// geo_weight_scale). X null: not G. sG: 6 P doubles of dynamic shared memory (if X). bad: bit 0 det J <= 0, bit 1
+// an element that fixed point rebuilds with less than FP64's precision. Bound by the FP64 pipe, as k_geometry is; exponents
+// are taken from the bits.
+__global__ void k_fixed_factors(const __grid_constant__ GllAll tab, int Np, int sw, const double* __restrict__ coef,
+                                const __grid_constant__ GeometryOut out, int2* __restrict__ X, int* __restrict__ gexp,
+                                GeoElement* __restrict__ geo, int* __restrict__ bad) {
   extern __shared__ double sG[];
-  __shared__ int sTop;
+  // largest exponents (as frexp has them) of |c_0|, |c_1|, |c_2| and their slopes, of G 2^(c_a + c_b) and of
+  // G 2^(c_0 + c_1 + c_2); the smallest of det J
+  __shared__ int sMax[5], sMin;
   const int P = Np * Np * Np;
   const int64_t e = blockIdx.x;
-  if (threadIdx.x == 0) sTop = -4000;
+  const double* a = coef + e * 24;
+  if (threadIdx.x < 5) sMax[threadIdx.x] = -4000;
+  if (threadIdx.x == 0) sMin = 4000;
   __syncthreads();
-  int top = -4000;
+  int most[5] = {-4000, -4000, -4000, -4000, -4000}, least = 4000;
+  auto exponent = [](double v) {
+    const int ex = (__double2hiint(v) >> 20) & 0x7ff;
+    return ex == 0 || ex == 0x7ff ? -4000 : ex - 1022;
+  };
+  // of a bound that rounding may have put below a power of two it reaches: the high word one up
+  auto exponent_up = [&](double v) { return exponent(__hiloint2double(__double2hiint(v) + 1, 0)); };
   for (int r = threadIdx.x; r < P; r += blockDim.x) {
     const int i = r % Np, j = (r / Np) % Np, k = r / (Np * Np);
-    double G[6], B, det;
-    point_geometry(coef + e * 24, tab.xi[i], tab.xi[j], tab.xi[k], tab.w[i] * tab.w[j] * tab.w[k], G, &B, &det);
+    const double wq = tab.w[i] * tab.w[j] * tab.w[k];
+    double G[6], det;
+    point_cofactors(a, tab.xi[i], tab.xi[j], tab.xi[k], G, &det);
     if (!(det > 0.0) || !isfinite(det)) atomicOr(bad, 1);
+    least = min(least, exponent(__hiloint2double(__double2hiint(det) - 1, 0)));
+    for (int d = 0; d < 3; ++d) {
+      const int ex = exponent_up(G[d == 0 ? 0 : d == 1 ? 3 : 5]);  // |c|^2 < 2^ex
+      most[d] = max(most[d], ex <= -4000 ? ex : (ex + 1) >> 1);
+    }
+    const double sc = wq / det;
     const int c[3] = {fixed_row_scale(Np, i), fixed_row_scale(Np, j), fixed_row_scale(Np, k)};
     for (int m = 0; m < 6; ++m) {
-      const double g = scalbn(G[m], c[m < 3 ? 0 : m < 5 ? 1 : 2] + c[m < 3 ? m : m < 5 ? m - 2 : 2]);
-      sG[m * P + r] = g;
-      int ex = -4000;
-      if (g != 0.0 && isfinite(g)) frexp(g, &ex);
-      top = max(top, ex);
+      G[m] = sc * G[m];
+      const int ca = c[m < 3 ? 0 : m < 5 ? 1 : 2] + c[m < 3 ? m : m < 5 ? m - 2 : 2];
+      most[3] = max(most[3], exponent(G[m]) + ca);
+      most[4] = max(most[4], exponent_up(G[m]) + c[0] + c[1] + c[2]);
+      if (X) sG[m * P + r] = exponent(G[m]) > -4000 ? __hiloint2double(__double2hiint(G[m]) + (ca << 20), __double2loint(G[m])) : 0.0;
     }
+    out.put(e, P, r, G, wq * det, sc);
   }
-  atomicMax(&sTop, top);
+  for (int q = threadIdx.x; q < 3 * Np; q += blockDim.x) {  // 4 P x K and 4 K x M of row q % 3, node q / 3
+    const int d = q % 3, p0 = d == 0 ? 2 : d == 1 ? 3 : 1, p1 = d == 0 ? 4 : d == 1 ? 6 : 5, m0 = d == 0 ? 3 : d == 1 ? 1 : 2,
+              m1 = d == 0 ? 5 : d == 1 ? 4 : 6, k0 = d == 0 ? 6 : d == 1 ? 5 : 4;
+    double p[3], m[3], k[3], v[3];
+    for (int c = 0; c < 3; ++c) {
+      const double xi = tab.xi[q / 3];
+      p[c] = a[3 * p0 + c] + a[3 * p1 + c] * xi;
+      m[c] = a[3 * m0 + c] + a[3 * m1 + c] * xi;
+      k[c] = a[3 * k0 + c] + a[21 + c] * xi;
+    }
+    int ex = -4000;
+    cross3(p, k, v);
+    for (int c = 0; c < 3; ++c) ex = max(ex, exponent_up(v[c]) + 2);
+    cross3(k, m, v);
+    for (int c = 0; c < 3; ++c) ex = max(ex, exponent_up(v[c]) + 2);
+    for (int r = 0; r < 3; ++r)
+      if (r == d) most[r] = max(most[r], ex);
+  }
+  for (int m = 0; m < 5; ++m) atomicMax(&sMax[m], most[m]);
+  atomicMin(&sMin, least);
   __syncthreads();
-  const int sg = 59 - sTop;
+  const int sg = 59 - sMax[3];
+  if (threadIdx.x == 0) {
+    double size = 0.0;
+    for (int c = 0; c < 3; ++c) {
+      double t = 0.0;
+      for (int m = 1; m < 8; ++m) t += fabs(a[3 * m + c]);
+      size = fmax(size, t);
+    }
+    const int row[3] = {sMax[0], sMax[1], sMax[2]};
+    GeoElement g;
+    const int qa = geo_scale(g, exponent_up(size), row, sMin, sMax[3], sMax[4], sw);
+    for (int m = 0; m < 7; ++m)
+      for (int c = 0; c < 3; ++c) g.a[m][c] = geo_fixed(a[3 * m + 3 + c], qa);
+    geo[e] = g;
+    if (g.sg == kGeoNone) atomicOr(bad, 2);
+    if (gexp) gexp[e] = sg;
+  }
+  if (!X) return;
   for (int q = threadIdx.x; q < 6 * P; q += blockDim.x) {
-    const long long x = __double2ll_rn(scalbn(sG[q], sg));
+    const long long x = (geo_fixed(sG[q], sg + 1) + 1) >> 1;  // rounded
     const int lo = static_cast<int>(static_cast<uint32_t>(x));
     X[e * 6 * P + q] = make_int2(lo, static_cast<int>((x - lo) >> 32));
   }
-  if (threadIdx.x == 0) gexp[e] = sg;
 }
 
 __global__ void k_coords(const __grid_constant__ GllAll tab, int Np, int64_t E, const double* __restrict__ coef,
@@ -383,23 +462,21 @@ sem_status launch_coefficients(int64_t E, const double* X, double* coef64, float
 
 sem_status launch_geometry(int N, int64_t E, const double* coef64, double* G64, float* G32, double* B64, float* B32,
                            int* bad, int64_t gs64, int64_t gs32, cudaStream_t s, double* S64, float* S32,
-                           float* GX) {
-  const int Np = N + 1;
-  const int64_t n = E * Np * Np * Np;
-  k_geometry<<<ceil_div(n, kThreads), kThreads, 0, s>>>(gll_all(N), Np, E, coef64, G64, G32, B64, B32, bad, gs64,
-                                                        gs32, S64, S32, GX);
-  count_launch();
-  SEM_CUDA_TRY(cudaGetLastError());
-  return SEM_OK;
-}
-
-sem_status launch_fixed_factors(int N, int64_t E, const double* coef64, int2* X, int* gexp, int* bad, cudaStream_t s) {
-  const int P = (N + 1) * (N + 1) * (N + 1);
-  static const cudaError_t attr = cudaFuncSetAttribute(k_fixed_factors, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       6 * kMaxNp * kMaxNp * kMaxNp * static_cast<int>(sizeof(double)));
-  SEM_CUDA_TRY(attr);
-  k_fixed_factors<<<static_cast<unsigned>(E), P < 128 ? 64 : P < 600 ? 128 : 256, 6 * static_cast<size_t>(P) * sizeof(double), s>>>(
-      gll_all(N), N + 1, coef64, X, gexp, bad);
+                           float* GX, int2* X, int* gexp, GeoElement* geo) {
+  const int Np = N + 1, P = Np * Np * Np;
+  const GeometryOut out{G64, G32, B64, B32, gs64, gs32, S64, S32, GX};
+  if (geo) {
+    int c[kMaxNp];
+    for (int i = 0; i < Np; ++i) c[i] = fixed_row_scale(Np, i);
+    static const cudaError_t attr = cudaFuncSetAttribute(k_fixed_factors, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                         6 * kMaxNp * kMaxNp * kMaxNp * static_cast<int>(sizeof(double)));
+    SEM_CUDA_TRY(attr);
+    k_fixed_factors<<<static_cast<unsigned>(E), P < 128 ? 64 : P < 600 ? 128 : 256,
+                      X ? 6 * static_cast<size_t>(P) * sizeof(double) : 0, s>>>(
+        gll_all(N), Np, geo_weight_scale(gll_table(N).w, c, Np), coef64, out, X, gexp, geo, bad);
+  } else {
+    k_geometry<<<ceil_div(E * P, kThreads), kThreads, 0, s>>>(gll_all(N), Np, E, coef64, out, bad);
+  }
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "../../include/sem.h"
+#include "k_geo_fixed.cuh"
 
 namespace sem {
 
@@ -133,12 +134,13 @@ inline int64_t factor_stride(int Np, bool fp32) {
   return fp32 ? (s + 3) / 4 * 4 : s;
 }
 
-// Orders whose FP64 stored-factor operator runs on the tensor cores (k_ax_slice.cuh, k_ax_slice16.cuh).
+// Orders whose FP64 operator runs on the tensor cores (k_ax_slice.cuh, k_ax_slice16.cuh): with stored factors, and on
+// the fly on meshes whose elements fixed point rebuilds as exactly as FP64 (sem_mesh_s::geo).
 // Their meshes keep G as 64-bit fixed point instead of FP64, in the same bytes: X = G_ab 2^(sg + c_a + c_b),
 // |X| <= 2^59, as 32-bit signed halves (low, high), with sg per element and c = fixed_row_scale of the
-// point's index along each direction. At 16.8M points the FP64 kernel against this one: N = 3 1.12 and
+// point's index along each direction. Stored, at 16.8M points the FP64 kernel against this one: N = 3 1.12 and
 // 0.36 ms, N = 5 1.50 and 0.75, N = 6 1.52 and 0.59, N = 7 1.50 and 0.34, N = 9 2.03 and 1.51, N = 10 1.79 and
-// 1.08, N = 11 2.06 and 0.85. N = 2, 4 and 8 fill too little of the boxes of 8 or 16 points a side that the
+// 1.08, N = 11 2.06 and 0.85; on the fly 1.7 to 2.9 times (k_ax_slice.cuh). N = 2, 4 and 8 fill too little of the boxes of 8 or 16 points a side that the
 // tensor cores work on (N = 2 0.86 against 0.93 ms, N = 4 1.13 against 1.31; 729 of 2304 points at N = 8). At
 // N = 1 the FP64 differences of equal values are exact zeros, which fixed-point factors do not keep on
 // stretched elements (relative error 1.4e-15 against 1.2e-16 at aspect ratio 100).
@@ -244,6 +246,7 @@ struct sem_mesh_s {
   double* G64 = nullptr;      // [E][6][P] or null (ax_slice_order: only for fewer elements than SMs)
   int2* GI = nullptr;         // [E][6][P] fixed-point factors (ax_slice_order; at N = 7 for SEM_F64X too) or null
   int* gexp = nullptr;        // [E] their exponents sg
+  sem::GeoElement* geo = nullptr;  // [E] elements for factors rebuilt in fixed point (ax_slice_order), or null: not this mesh
   float* G32 = nullptr;       // [E][factor_stride] (the [6][P] block, padded to 16 bytes) or null
   float* Gx = nullptr;        // [E][6][P] float pairs (high, low) of G for SEM_F64X (but f64x_on_slices), or null
   double* scale64 = nullptr;  // [n] w_i w_j w_k / det J (SEM_MESH_OTF_SCALE) or null
@@ -296,6 +299,7 @@ struct AxLaunch {
   const void* G;      // stored factors or null
   bool g_pairs;       // SEM_F64X: G holds float pairs (high, low) instead of the FP64 operator's factors
   const int* gexp;    // exponents of fixed-point factors (ax_slice_order)
+  const GeoElement* geo;  // elements for fixed-point factors rebuilt on the fly, or null
   const void* coef;   // trilinear coefficients (otf)
   const void* scale;  // per-point w/det J (otf with stored scale)
   // CG mode (p = z + beta p prologue, <p, w> partials in the epilogue)
@@ -320,8 +324,12 @@ sem_status launch_ax_f32_hi(int N, sem_ax_variant v, bool cg_mode, const AxLaunc
 // FP64 with stored (fixed-point) factors on the tensor cores, ax_slice_order only.
 sem_status launch_ax_slice(int N, bool cg_mode, const AxLaunch& a, cudaStream_t s);
 sem_status launch_ax_slice_hi(int N, bool cg_mode, const AxLaunch& a, cudaStream_t s);  // N + 1 >= 9
+// The same with the factors rebuilt on the fly (a.geo).
+sem_status launch_ax_slice_otf(int N, bool cg_mode, const AxLaunch& a, cudaStream_t s);
+sem_status launch_ax_slice_otf_hi(int N, bool cg_mode, const AxLaunch& a, cudaStream_t s);
 inline sem_status launch_ax_f64(int N, sem_ax_variant v, bool cg, const AxLaunch& a, cudaStream_t s) {
   if (v == SEM_AX_STORED && ax_slice_order(N)) return launch_ax_slice(N, cg, a, s);
+  if (v != SEM_AX_STORED && a.geo) return launch_ax_slice_otf(N, cg, a, s);
   return N + 1 <= 7 ? launch_ax_f64_lo(N, v, cg, a, s) : launch_ax_f64_hi(N, v, cg, a, s);
 }
 inline sem_status launch_ax_f32(int N, sem_ax_variant v, bool cg, const AxLaunch& a, cudaStream_t s) {
@@ -372,12 +380,13 @@ sem_status launch_probe_barrier(unsigned* bar, int blocks, int skip_block, int* 
 
 // element geometry (k_mesh.cu)
 sem_status launch_coefficients(int64_t E, const double* X, double* coef64, float* coef32, cudaStream_t s);
-// G64 / G32 (either may be null) are written with element strides gs64 / gs32.
+// G64 / G32 (either may be null) are written with element strides gs64 / gs32. geo (ax_slice_order): also the
+// fixed-point factors X with their exponents (null: not those) and the elements of factors rebuilt on the fly.
+// bad_flag: bit 0 det J <= 0 somewhere, bit 1 geo is not for this mesh.
 sem_status launch_geometry(int N, int64_t E, const double* coef64, double* G64, float* G32, double* B64,
                            float* B32, int* bad_flag, int64_t gs64, int64_t gs32, cudaStream_t s,
-                           double* S64 = nullptr, float* S32 = nullptr, float* GX = nullptr);
-// Fixed-point factors and their exponents (ax_slice_order), with the det J > 0 check.
-sem_status launch_fixed_factors(int N, int64_t E, const double* coef64, int2* X, int* gexp, int* bad_flag, cudaStream_t s);
+                           double* S64 = nullptr, float* S32 = nullptr, float* GX = nullptr,
+                           int2* X = nullptr, int* gexp = nullptr, GeoElement* geo = nullptr);
 sem_status launch_coords(int N, int64_t E, const double* coef64, double* xyz, int64_t n, cudaStream_t s);
 sem_status launch_local_diag(int N, int64_t E, const double* coef64, double* d, cudaStream_t s);
 sem_status launch_rhs_local(int N, int64_t E, const double* coef64, int a, int b, int c, double* out,
@@ -396,8 +405,8 @@ inline bool cg_layout(sem_prec prec) { return prec != SEM_F32; }
 // The FP32, double-float and tensor-core FP64 operators take the fused CG prologue (AxLaunch::r, minv,
 // x): the update kernel then skips x and z, and after the last iteration launch_cg_flush adds the
 // pending alpha p. The FP64-pipe-bound k_ax leaves both to the update kernel.
-inline bool fused_cg(sem_prec prec, int N, sem_ax_variant v) {
-  return prec != SEM_F64 || (v == SEM_AX_STORED && ax_slice_order(N));
+inline bool fused_cg(sem_prec prec, int N, sem_ax_variant v, const GeoElement* geo) {
+  return prec != SEM_F64 || (v == SEM_AX_STORED ? ax_slice_order(N) : geo != nullptr);
 }
 sem_status launch_dssum_cg(sem_prec prec, const GsPlan& g, void* w, CgScalars* st, const double* ax_partials,
                            int ax_blocks, cudaStream_t s);
