@@ -173,15 +173,22 @@ __host__ __device__ constexpr int ax_gstride() {
   return sizeof(T) == 8 ? 6 * NP * NP * NP : (6 * NP * NP * NP + 3) / 4 * 4;
 }
 
-// Staging buffer of one element in shared memory: position of point (i, j, k). For NP = 8
-// every k-plane has one row of padding and the position inside a row is XOR-swizzled by
-// (j >> 1) | ((k & 1) << 2); then the three access patterns of k_ax (a thread per i-row, a
-// thread per j-line, a thread per k-column, 32 consecutive threads covering four rows, lines
-// or columns) touch every shared-memory bank equally often, for FP64 and FP32 data.
+// Staging buffer of one element in shared memory: position of point (i, j, k). Three patterns use it, 32
+// consecutive threads (16 for 8-byte values) of a block at a time: a thread per k-column (7 accesses
+// per point of k_ax's plain mode), per i-row (4) and per j-line (4), and in FP32 with stored factors these accesses
+// bound the kernel next to HBM (N = 5: 80% of the shared-memory wavefronts, 71% of the bandwidth). The plane stride
+// kPlane and the element stride kSize are those with the fewest bank conflicts over the three where that
+// pays: wavefronts per 32 points unpadded and so, and FP32 A_L stored at 16.8M points: N = 3 46 and 19, 106.7 and
+// 84.7 us (on the fly 94.9 and 86.2); N = 5 26.4 and 21.4, 94.2 and 90.4 us; N = 6 one element per block 21 and 19,
+// 94.3 and 90.7 us. At N = 1, 9 and 11 fewer conflicts (30 and 19, 24 and 21, 28.6 and 22.2) change nothing, at N = 11 on the
+// fly the larger buffers cost 4%; at the other orders no padding helps. For NP = 8 the position inside a row is
+// XOR-swizzled by (j >> 1) | ((k & 1) << 2) besides, and no pattern has conflicts.
+// kSize is even where N + 1 is: TMA targets that follow stay 16-byte aligned.
 template <int NP>
 struct Stage {
-  static constexpr int kPlane = NP == 8 ? 72 : NP * NP;
-  static constexpr int kSize = NP * kPlane;
+  static constexpr int kPlane =
+      NP == 4 ? 19 : NP == 6 ? 43 : NP == 7 ? 52 : NP == 8 ? 72 : NP * NP;
+  static constexpr int kSize = NP == 4 ? 80 : NP == 6 ? 260 : NP * kPlane;
   __device__ static __forceinline__ int at(int i, int j, int k) {
     if constexpr (NP == 8)
       return k * kPlane + j * NP + (i ^ ((j >> 1) | ((k & 1) << 2)));
