@@ -36,7 +36,7 @@
 // On the fly (Section 5.1's rematerialised factors) the same kernel fills its factor buffer from the element's
 // coefficients, with about 700 instructions per point on the same pipes, still far below the 45 FP64 instructions
 // of k_ax for it. A_L in ms, k_ax and this kernel, 16M points: N = 3 2.72 and 1.10, N = 5 3.07 and 1.60, N = 6 2.98 and
-// 1.45, N = 7 2.63 and 0.90, N = 9 3.62 and 2.09, N = 10 3.13 and 1.78, N = 11 3.49 and 1.50 (of these the factors take
+// 1.37, N = 7 2.63 and 0.90, N = 9 3.62 and 2.08, N = 10 3.13 and 1.78, N = 11 3.49 and 1.46 (of these the factors take
 // 0.5 ms, the row tables 0.05 and at N = 3 0.2); with the per-point scale of SEM_AX_OTF_SCALE, which is not read
 // here, 2.31, 2.67, 2.58, 2.30, 3.18, 2.75 and 3.15 before. Error against FP64 torch as with k_ax (N = 9 1.2e-15 and
 // 1.3e-15, N = 7 9.0e-16 and 9.3e-16).
@@ -409,11 +409,15 @@ struct OtfFactors {
 };
 
 // On the fly: the row tables of one group's elements in shared memory, and the group's factors from
-// them (k_geo_fixed.cuh). THREADS threads take kParts parts of every k-column.
+// them (k_geo_fixed.cuh). THREADS threads take kParts parts of every k-column, or points.
 template <int NP, int ELEMS, int THREADS>
 struct OtfGeometry {
   static constexpr int NP2 = NP * NP, P = NP2 * NP;
   static constexpr int kParts = THREADS / (ELEMS * NP2) > 1 ? THREADS / (ELEMS * NP2) : 1;
+  // Point by point (each sets its column up again) where that takes fewer rounds of the block and measures faster:
+  // A_L at 16M points by columns and by points, N = 6 (four and three rounds) 1.45 and 1.37 ms, N = 11 (six and five)
+  // 1.50 and 1.46; but N = 10 (six and four) 1.78 and 1.83, and at the other orders the rounds are the same.
+  static constexpr bool kByPoint = NP != 11 && (ELEMS * P + THREADS - 1) / THREADS < (NP + kParts - 1) / kParts;
   struct Tables {
     GeoEntry e[ELEMS][3][NP][3];
     GeoEntryT t[ELEMS][NP][3];
@@ -442,23 +446,33 @@ struct OtfGeometry {
   static __device__ __forceinline__ void columns(const Tables* s, const GeoElement* __restrict__ geo, int64_t e0, int count,
                                                  int2* sG) {
     const int one = one_of(s);
-    for (int q = threadIdx.x; q < NP2 * kParts * count; q += THREADS) {
-      const int el = q / (NP2 * kParts), part = q / NP2 % kParts, col = q % NP2, i = col % NP, j = col / NP;
+    auto column = [&](int el, int i, int j, int k0, int k1) {
       const GeoEntry *e_i = s->e[el][0][i], *e_j = s->e[el][1][j];
       const int down = __ldg(&geo[e0 + el].down), lz = __ldg(&geo[e0 + el].lz);
       const int up = __ldg(&geo[e0 + el].up) & 255, b = __ldg(&geo[e0 + el].up) >> 8;
       GeoColumn c;
       c.init(e_i, e_j, s->t[el][i], s->n.x[i], s->n.x[j], s->n.w[i], s->n.w[j], one);
       const int ci = fixed_row_scale(NP, i), cj = fixed_row_scale(NP, j);
-      int2* out = sG + el * 6 * P + col;
+      int2* out = sG + el * 6 * P + j * NP + i;
 #pragma unroll 1
-      for (int k = part * NP / kParts; k < (part + 1) * NP / kParts; ++k) {
+      for (int k = k0; k < k1; ++k) {
         const int ck = fixed_row_scale(NP, k);
         const int sh[6] = {b + cj + ck - ci, b + ck, b + cj, b + ci + ck - cj, b + ci, b + ci + cj - ck};
         c.point(e_i, e_j, s->e[el][2][k], s->n.x[k], s->n.w[k], down, lz, up, [&](int m, long long v) {
           const Fx x = fx_split(v >> sh[m]);
           out[m * P + k * NP2] = make_int2(x.l, x.h);
         });
+      }
+    };
+    if constexpr (kByPoint) {
+      for (int q = threadIdx.x; q < P * count; q += THREADS) {
+        const int el = q / P, k = q % P / NP2;
+        column(el, q % NP, q % NP2 / NP, k, k + 1);
+      }
+    } else {
+      for (int q = threadIdx.x; q < NP2 * kParts * count; q += THREADS) {
+        const int el = q / (NP2 * kParts), part = q / NP2 % kParts;
+        column(el, q % NP2 % NP, q % NP2 / NP, part * NP / kParts, (part + 1) * NP / kParts);
       }
     }
   }
