@@ -94,8 +94,9 @@ __device__ __forceinline__ void gs_class(const GsPlan& g, int c, int64_t t0, int
   }
 }
 
-template <typename T>
-__global__ void k_dssum(const GsPlan g, T* __restrict__ u, int apply_mask) {
+// MINB: blocks per SM whose registers the compiler has to leave (launch_dssum).
+template <typename T, int MINB>
+__global__ void __launch_bounds__(kThreads, MINB) k_dssum(const GsPlan g, T* __restrict__ u, int apply_mask) {
   const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   auto value = [&](bool masked, T sum) { return (apply_mask && masked) ? T(0) : sum; };
@@ -186,10 +187,15 @@ __global__ void k_dssum_invert(const GsPlan g, const double* __restrict__ d, dou
 sem_status launch_dssum(sem_prec prec, const GsPlan& g, void* u, int apply_mask, cudaStream_t s) {
   if (g.total() == 0) return SEM_OK;
   const int grid = seg_grid(g.total());
-  if (prec == SEM_F64)
-    k_dssum<double><<<grid, kThreads, 0, s>>>(g, static_cast<double*>(u), apply_mask);
+  // FP64: four blocks per SM where segments of two copies (faces) are most of the work, the compiler's choice of
+  // registers (three blocks) where those of four need them: us without and with four, N = 5 (48 faces' segments to 12
+  // edges' per element) 72.3 and 67.5, N = 7 72.5 and 65.3, N = 9 32.5 and 27.8, but N = 3 (12 to 6) 81.8 and 86.0
+  if (prec == SEM_F64 && g.n[1] >= 3 * g.n[2])
+    k_dssum<double, 4><<<grid, kThreads, 0, s>>>(g, static_cast<double*>(u), apply_mask);
+  else if (prec == SEM_F64)
+    k_dssum<double, 1><<<grid, kThreads, 0, s>>>(g, static_cast<double*>(u), apply_mask);
   else
-    k_dssum<float><<<grid, kThreads, 0, s>>>(g, static_cast<float*>(u), apply_mask);
+    k_dssum<float, 1><<<grid, kThreads, 0, s>>>(g, static_cast<float*>(u), apply_mask);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;
