@@ -94,7 +94,7 @@ __device__ __forceinline__ void gs_class(const GsPlan& g, int c, int64_t t0, int
   }
 }
 
-// MINB: blocks per SM whose registers the compiler has to leave (launch_dssum).
+// MINB: blocks per SM whose registers the compiler has to leave, 0: its own choice (launch_dssum).
 template <typename T, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k_dssum(const GsPlan g, T* __restrict__ u, int apply_mask) {
   const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -193,9 +193,9 @@ sem_status launch_dssum(sem_prec prec, const GsPlan& g, void* u, int apply_mask,
   if (prec == SEM_F64 && g.n[1] >= 3 * g.n[2])
     k_dssum<double, 4><<<grid, kThreads, 0, s>>>(g, static_cast<double*>(u), apply_mask);
   else if (prec == SEM_F64)
-    k_dssum<double, 1><<<grid, kThreads, 0, s>>>(g, static_cast<double*>(u), apply_mask);
+    k_dssum<double, 0><<<grid, kThreads, 0, s>>>(g, static_cast<double*>(u), apply_mask);
   else
-    k_dssum<float, 1><<<grid, kThreads, 0, s>>>(g, static_cast<float*>(u), apply_mask);
+    k_dssum<float, 0><<<grid, kThreads, 0, s>>>(g, static_cast<float*>(u), apply_mask);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;
