@@ -64,7 +64,8 @@ typedef enum {
  * SEM_MESH_F64X_STORED if the mesh has them, else the FP64 ones; with SEM_AX_OTF on factors
  * rebuilt from the element's trilinear coefficients (the per-column polynomial coefficients
  * in FP64, every point in double-float); SEM_AX_OTF_SCALE gives SEM_ERR_UNSUPPORTED. At orders 7 and 11
- * SEM_AX_STORED is the operator of SEM_F64, which is the faster one there. Every other call treats
+ * SEM_AX_STORED is the operator of SEM_F64, which is the faster one there (but for sem_ax at order 7 on
+ * meshes of fewer than 2560 elements). Every other call treats
  * SEM_F64X like SEM_F64. Values below 2^-126 in magnitude are flushed to zero inside it. */
 typedef enum { SEM_F64 = 0, SEM_F32 = 1, SEM_F64X = 2 } sem_prec;
 
@@ -88,7 +89,8 @@ typedef enum { SEM_AX_STORED = 0, SEM_AX_OTF = 1, SEM_AX_AUTO = 2, SEM_AX_OTF_SC
 #define SEM_MESH_OTF_SCALE 4u  /* w_i w_j w_k / det J per point, FP64 and FP32: 12 bytes per local point */
 #define SEM_MESH_F64X_STORED 8u /* G as float pairs (high, low: 48 significant bits) for SEM_F64X: 48 bytes
                                  * per local point; without it SEM_F64X splits the FP64 factors itself (orders 7, 11: the array
-                                 * of SEM_MESH_F64_STORED, held once) */
+                                 * of SEM_MESH_F64_STORED, held once; order 7 below 2560 elements
+                                 * the float pairs too) */
 
 typedef struct sem_mesh_s* sem_mesh;
 typedef struct sem_cg_s* sem_cg;

@@ -214,6 +214,10 @@ sem_status launch_ax_any(sem_mesh m, sem_prec prec, sem_ax_variant v, bool cg, A
   const bool fp64_data = prec != SEM_F32;
   a.coef = fp64_data ? static_cast<const void*>(m->coef64) : static_cast<const void*>(m->coef32);
   a.G = stored_factors(m, prec, &a.g_pairs);
+  if (cg && a.g_pairs && f64x_on_slices(m->N)) {  // (the pairs are for the plain operator, f64x_plain_pairs)
+    a.G = m->GI;
+    a.g_pairs = false;
+  }
   a.gexp = m->gexp;
   a.geo = m->geo;
   a.scale = fp64_data ? static_cast<const void*>(m->scale64) : static_cast<const void*>(m->scale32);
@@ -372,7 +376,7 @@ extern "C" sem_status sem_mesh_create(int N, int64_t nv, const double* vert_xyz,
       SEM_STEP(dmalloc(&m->gexp, static_cast<size_t>(E), &acc, s));
     }
     if (ax_slice_order(N)) SEM_STEP(dmalloc(&m->geo, static_cast<size_t>(E), &acc, s));
-    if ((flags & SEM_MESH_F64X_STORED) && !x_fixed)
+    if ((flags & SEM_MESH_F64X_STORED) && (!x_fixed || f64x_plain_pairs(N, E)))
       SEM_STEP(dmalloc(&m->Gx, static_cast<size_t>(2 * E * 6 * P), &acc, s));
     if (flags & SEM_MESH_F32_STORED)
       SEM_STEP(dmalloc(&m->G32, static_cast<size_t>(E * factor_stride(m->Np, true)), &acc, s));
@@ -855,7 +859,7 @@ sem_status cg_start(sem_cg c, const void* b, void* x, bool x0_is_zero, cudaStrea
     // f64x_on_slices both are the same operator.)
     sem_prec rp = c->prec;
     sem_ax_variant rv = c->variant;
-    if (rp == SEM_F64X && !(rv == SEM_AX_STORED && f64x_on_slices(m->N))) {
+    if (rp == SEM_F64X && !(rv == SEM_AX_STORED && f64x_on_slices(m->N) && !m->Gx)) {
       rp = SEM_F64;
       if (rv == SEM_AX_STORED && !has_factors(m, SEM_F64)) rv = SEM_AX_OTF;
     }

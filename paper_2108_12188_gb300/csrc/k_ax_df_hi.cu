@@ -9,6 +9,8 @@ template <int NP>
 struct DfStored {
   static sem_status run(int N, bool cg, const AxLaunch& a, cudaStream_t s) {
     if constexpr (f64x_on_slices(NP - 1)) {
+      if constexpr (f64x_plain_pairs(NP - 1, 0))
+        if (a.g_pairs && !cg) return launch_df_t<NP, false, kGkPairs>(N, a, s);
       return launch_ax_slice(N, cg, a, s);
     } else {
       if (a.g_pairs)

@@ -150,6 +150,11 @@ __host__ __device__ constexpr bool ax_slice_order(int N) { return N == 3 || (N >
 // 0.643; N = 11 0.92 and 1.20, 1.31 and 1.95; but N = 3 0.36 and 0.27, N = 5 0.79 and 0.38, N = 6 0.62 and
 // 0.50, N = 9 1.45 and 0.73, N = 10 1.13 and 0.71).
 __host__ __device__ constexpr bool f64x_on_slices(int N) { return N == 7 || N == 11; }
+// The plain operator (sem_ax) keeps double-float factors for meshes of fewer elements than this at N = 7: its blocks
+// take two elements and fill one or two waves where the slices take two or three. Slices and double-float in us:
+// 1000 elements 22.6 and 16.5, 1728 28.8 and 24.8, 2744 38.9 and 39.7, 4096 53.9 and 59.8 (a CG iteration is faster on the
+// slices at every size).
+constexpr bool f64x_plain_pairs(int N, int64_t E) { return N == 7 && E < 2560; }
 __host__ __device__ constexpr int fixed_row_scale(int NP, int i) {
   return i == 0 || i == NP - 1 ? (NP <= 4 ? 1 : 2) : 0;
 }
@@ -248,7 +253,7 @@ struct sem_mesh_s {
   int* gexp = nullptr;        // [E] their exponents sg
   sem::GeoElement* geo = nullptr;  // [E] elements for factors rebuilt in fixed point (ax_slice_order), or null: not this mesh
   float* G32 = nullptr;       // [E][factor_stride] (the [6][P] block, padded to 16 bytes) or null
-  float* Gx = nullptr;        // [E][6][P] float pairs (high, low) of G for SEM_F64X (but f64x_on_slices), or null
+  float* Gx = nullptr;        // [E][6][P] float pairs (high, low) of G for SEM_F64X (f64x_on_slices: only f64x_plain_pairs), or null
   double* scale64 = nullptr;  // [n] w_i w_j w_k / det J (SEM_MESH_OTF_SCALE) or null
   float* scale32 = nullptr;
   int32_t* gs_rec[sem::kGsClasses] = {};  // gather-scatter plan (views in gs)
