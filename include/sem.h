@@ -54,9 +54,12 @@ typedef enum {
 } sem_status;
 
 /* SEM_F64: FP64 data and arithmetic of FP64 accuracy: FP64 instructions, and for the operator at orders 3,
- * 5 to 7 and 9 to 11 exact integer products on the tensor cores with 64-bit fixed point (elements
- * that hold infinities, NaN or values near the ends of the FP64 range take FP64 instructions, and so do
- * meshes with elements so distorted that fixed point would lose precision on the fly). SEM_F32: FP32 data and arithmetic.
+ * 5 to 7 and 9 to 11 exact integer products on the tensor cores with 64-bit fixed point, relative to the largest values of
+ * an element. There the error of A_L u is of FP64's size in the 2-norm over an element (at most 1e-14 of
+ * |A_L| |u|, 2e-16 for values of one size), not value by value: where other values of the element are larger by 2^k, a value has
+ * the last k of 58 bits less. Elements that hold infinities, NaN or values near the ends of the FP64 range, or only a few values
+ * of the size of the largest, take FP64 instructions, and so do
+ * meshes with elements so distorted that fixed point would lose precision on the fly. SEM_F32: FP32 data and arithmetic.
  * SEM_F64X: FP64 data (double* vectors, FP64 stored factors); the local operator runs in
  * double-float arithmetic (pairs of floats with error-free products and sums, about 47
  * significant bits) on the FP32 pipes, which GB300 issues 64 times faster than FP64. Only

@@ -45,11 +45,10 @@
 // kernels against an 80-bit reference; k_ax in brackets): random u 8e-17 (1.8e-16), a sine over 8^3
 // elements 4e-16 (1.4e-14), one plus 1e-8 of a sine 5e-9 (1.2e-6), aspect ratio 100 4e-12 (5e-11),
 // exp(-3 (x + y + z)) over two elements 6e-16 (3.0e-15). Fixed point is relative to the element's
-// largest value: a field that falls by e^5 per element and direction, which N = 7 does not
-// resolve, has 1.5e-15 (7e-16).
+// largest value, and so is the error at every node, see kNear.
 //
 // Elements that fixed point does not take (an infinity or NaN, magnitudes within about 2^60 of the
-// ends of the FP64 range) run the FP64 lines of k_ax, in element_fp64.
+// ends of the FP64 range, few values near the largest, see kNear) run the FP64 lines of k_ax, in elements_fp64.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -332,81 +331,79 @@ __device__ __forceinline__ double to_double(long long v, int k) {
   return a ? __hiloint2double(static_cast<int>(h | sign), static_cast<int>(static_cast<uint32_t>(m))) : 0.0;
 }
 
-// The element in FP64, as k_ax computes it (lines through the even/odd split of D): w of the whole
-// element to out[0 .. NP^3). factors(q, g): the six factors of point q. scratch: 3 NP^3 doubles of shared
-// memory. Called by all threads.
-template <int NP, typename F>
-__device__ __noinline__ void element_fp64(const GllParam<NP, double>& tab, const double* __restrict__ u, const F& factors,
-                                          double* scratch, double* out) {
+// Fixed point is relative to the element's largest |u|: where only a few of an element's values come near it, the
+// others lose bits that FP64 keeps, so such an element takes FP64 lines. A thread's largest value counts if it is
+// within 2^kNear of its warp's and that within 2^kNearWarp of the element's (by exponent); fewer than a quarter of the threads
+// with points: FP64. Relative 2-norm error of w over an element, CPU model of both, 2000 fields with spikes, decays and ridges:
+// without this rule up to 3.5e-15 at N = 3, 4.9e-14 at N = 7, 1.8e-13 at N = 11 (FP64 lines 2e-16), with it at most 1.5e-15,
+// 2.5e-15 and 3.3e-15, on average as FP64. Random fields have 2e-16 either way; in CG with a smooth or a random right-hand
+// side 37% of the threads or more count in every element and iteration, with a point source a quarter is missed in the first
+// 12% of them. A_L in us at 4.1M points where every element takes FP64 lines, k_ax in brackets: N = 3 294 (282), N = 5 417 (344), N = 6
+// 412 (371), N = 7 371 (378), N = 9 595 (530), N = 10 558 (422), N = 11 570 (500); on the fly 414 (695), 522 (750), 543 (774), 462
+// (719), 770 (941), 703 (735), 707 (841). The rule itself, and u kept for such elements: N = 3 344 -> 354 us at 16.8M points, N = 7
+// 345 -> 335 and in CG 547 -> 554 an iteration, the other orders within 2%.
+constexpr int kNear = 4, kNearWarp = 3;
+
+// A warp's word on its values (or those of an element in it): the largest exponent above the number of threads within 2^kNear.
+__device__ __forceinline__ unsigned near_word(unsigned top, unsigned most, unsigned lanes) {
+  return (most & 0x7ff00000u) | __popc(__ballot_sync(0xffffffffu, (top >> 20) + kNear >= (most >> 20)) & lanes);
+}
+
+// `count` elements in FP64, as k_ax computes them (lines through the even/odd split of D). abc: the arrays A, B, C
+// of ELEMS NP^3 doubles each in shared memory; A holds u, and w = A + B + C on return. G: the elements' fixed-point factors in
+// shared memory, sg[q sg_step] the exponent of element q. Called by all threads after a barrier, ends with one.
+template <int NP, int ELEMS>
+__device__ __noinline__ void elements_fp64(const GllParam<NP, double>& tab, const int2* G, const int* __restrict__ sg,
+                                           int sg_step, int count, double* abc) {
   constexpr int NP2 = NP * NP, P = NP2 * NP;
-  double *A = scratch, *B = A + P, *C = B + P;
-  const int t = threadIdx.x, nt = blockDim.x;
-  auto lines = [&](const EoMat<NP, double>& M, const double* src, double* dst, int s0, int s1, int step) {
-    for (int q = t; q < NP2; q += nt) {
-      const int base = (q % NP) * s0 + (q / NP) * s1;
-      double in[NP], o[NP];
-      for (int l = 0; l < NP; ++l) in[l] = src[base + l * step];
-      eo_apply<NP, double>(M, in, o);
-      for (int l = 0; l < NP; ++l) dst[base + l * step] = o[l];
-    }
+  double *A = abc, *B = A + ELEMS * P, *C = B + ELEMS * P;
+  const int t = threadIdx.x, nt = blockDim.x, lines = count * NP2;
+  auto line = [&](const EoMat<NP, double>& M, const double* src, double* dst, int q, int dir) {
+    const int r = q % NP2, a = r % NP, b = r / NP;
+    const int base = q / NP2 * P + (dir == 0 ? (a + b * NP) * NP : dir == 1 ? a + b * NP2 : r);
+    const int step = dir == 0 ? 1 : dir == 1 ? NP : NP2;
+    double in[NP], o[NP];
+#pragma unroll
+    for (int l = 0; l < NP; ++l) in[l] = src[base + l * step];
+    eo_apply<NP, double>(M, in, o);
+#pragma unroll
+    for (int l = 0; l < NP; ++l) dst[base + l * step] = o[l];
   };
-  for (int q = t; q < P; q += nt) A[q] = __ldcg(u + q);  // CG: p, stored by this block in this launch
+#pragma unroll 1
+  for (int q = t; q < 2 * lines; q += nt) {
+    const bool rows = q < lines;
+    line(tab.Df, A, rows ? B : C, rows ? q : q - lines, rows ? 0 : 2);
+  }
   __syncthreads();
-  lines(tab.Df, A, B, NP, NP2, 1);   // i-rows
-  lines(tab.Df, A, C, 1, NP, NP2);   // k-columns
+#pragma unroll 1
+  for (int q = t; q < lines; q += nt) line(tab.Df, A, A, q, 1);
   __syncthreads();
-  lines(tab.Df, A, A, 1, NP2, NP);   // j-lines in place
-  __syncthreads();
-  for (int q = t; q < P; q += nt) {
+#pragma unroll 1
+  for (int q = t; q < count * P; q += nt) {
+    const int el = q / P, r = q % P, e = __ldg(sg + el * sg_step);
+    const int c[3] = {fixed_row_scale(NP, r % NP), fixed_row_scale(NP, r / NP % NP), fixed_row_scale(NP, r / NP2)};
     double g[6];
-    factors(q, g);
+#pragma unroll
+    for (int m = 0; m < 6; ++m) {
+      const int2 x = G[(el * 6 + m) * P + r];
+      const long long v = static_cast<long long>(x.y) * 4294967296ll + x.x;
+      const int k = -(e + c[m < 3 ? 0 : m < 5 ? 1 : 2] + c[m < 3 ? m : m < 5 ? m - 2 : 2]);
+      g[m] = abs(e) < 900 ? to_double(v, k) : scalbn(static_cast<double>(v), k);  // (to_double wants a normal result)
+    }
     const double ur = B[q], us = A[q], ut = C[q];
     B[q] = g[0] * ur + g[1] * us + g[2] * ut;
     A[q] = g[1] * ur + g[3] * us + g[4] * ut;
     C[q] = g[2] * ur + g[4] * us + g[5] * ut;
   }
   __syncthreads();
-  lines(tab.Dt, B, B, NP, NP2, 1);
-  lines(tab.Dt, A, A, 1, NP2, NP);
-  lines(tab.Dt, C, C, 1, NP, NP2);
-  __syncthreads();
-  for (int q = t; q < P; q += nt) out[q] = B[q] + A[q] + C[q];
+#pragma unroll 1
+  for (int q = t; q < 3 * lines; q += nt) {
+    const int dir = q / lines;
+    double* v = dir == 0 ? B : dir == 1 ? A : C;
+    line(tab.Dt, v, v, q - dir * lines, dir);
+  }
   __syncthreads();
 }
-
-// Its factors: fixed point (the element's block of G), or from the element's coefficients.
-template <int NP>
-struct StoredFactors {
-  const int2* G;
-  int sg;
-  __device__ __forceinline__ void operator()(int q, double (&g)[6]) const {
-    constexpr int NP2 = NP * NP, P = NP2 * NP;
-    const int c[3] = {fixed_row_scale(NP, q % NP), fixed_row_scale(NP, q / NP % NP), fixed_row_scale(NP, q / NP2)};
-    for (int m = 0; m < 6; ++m) {
-      const int ra = m < 3 ? 0 : m < 5 ? 1 : 2, rb = m < 3 ? m : m < 5 ? m - 2 : 2;
-      const int2 x = G[m * P + q];
-      const long long v = static_cast<long long>(x.y) * 4294967296ll + x.x;
-      g[m] = scalbn(static_cast<double>(v), -(sg + c[ra] + c[rb]));
-    }
-  }
-};
-template <int NP>
-struct OtfFactors {
-  const GllParam<NP, double>& tab;
-  const double* coef;
-  __device__ __forceinline__ void operator()(int q, double (&g)[6]) const {
-    constexpr int NP2 = NP * NP;
-    const int i = q % NP, j = q / NP % NP, k = q / NP2;
-    OtfColumn<double> geo;
-    geo.init(coef, tab.xi[i], tab.xi[j]);
-    const double gam = tab.xi[k], sc = tab.w[i] * tab.w[j] * tab.w[k] / geo.det(gam);
-    for (int a = 0; a < 3; ++a) {
-      double v[3] = {a == 0 ? 1.0 : 0.0, a == 1 ? 1.0 : 0.0, a == 2 ? 1.0 : 0.0};
-      geo.apply(gam, sc, v[0], v[1], v[2]);
-      for (int b = a; b < 3; ++b) g[a == 0 ? b : a + b + 1] = v[b];
-    }
-  }
-};
 
 // On the fly: the row tables of one group's elements in shared memory, and the group's factors from
 // them (k_geo_fixed.cuh). THREADS threads take kParts parts of every k-column, or points.
@@ -506,12 +503,16 @@ struct SliceShape {
   static constexpr size_t kBytesG = (kElems * static_cast<size_t>(kElemBytes) + 127) / 128 * 128;
   static constexpr size_t kOffD = kBytesG;                         // digits [kSlices][8][72] FP16
   static constexpr size_t kOffX = kOffD + kSlices * kDigit * 2;    // exchange [8][72] 64-bit
-  static constexpr size_t kOffA = kOffX + 8 * kPlane * 8;          // A fragments [2][4][32] 16 bytes
+  // (the digits and the exchange together also hold the three arrays of elements_fp64)
+  static constexpr size_t kBytesDX = kSlices * kDigit * 2 + 8 * kPlane * 8, kBytes64 = 24ull * kElems * NP * NP * NP;
+  static constexpr size_t kOffA = kOffD + (kBytes64 > kBytesDX ? kBytes64 : kBytesDX);  // A fragments [2][4][32] 16 bytes
   static constexpr size_t kOffB = kOffA + 2 * 4 * 32 * 16;         // B fragments [2][7][32] 8 bytes
   static constexpr size_t kOffC = kOffB + 2 * 7 * 32 * 8;          // Start
   static constexpr size_t kOffM = kOffC + 32;                      // maxima [3][kElems][kSlots]
   static constexpr size_t kOffBar = kOffM + (3 * kElems * kSlots * 4 + 7) / 8 * 8;
   static constexpr size_t kOffTab = (kOffBar + 8 + 15) / 16 * 16;  // on the fly: row tables
+  static constexpr int kHolders = NP * ((NP + 1) / 2) * ((NP + 1) / 2);  // threads with points of one element
+  static constexpr int kFew = (kHolders + 3) / 4;  // see kNear
   using Geometry = OtfGeometry<NP, kElems, kThreads>;
   static constexpr size_t bytes(bool otf) { return otf ? kOffTab + sizeof(typename Geometry::Tables) : kOffBar + 8; }
 };
@@ -544,7 +545,7 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, OTF && NP != 6 ? 3 :
     k_ax_slice(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab<NP> sl,
                const __grid_constant__ GeoNodes<NP> nodes, int64_t E, const double* __restrict__ u,
                double* __restrict__ w, const int2* __restrict__ G, const int* __restrict__ gexp,
-               const double* __restrict__ coef, const GeoElement* __restrict__ geo, const double* __restrict__ r, const double* __restrict__ minv,
+               const GeoElement* __restrict__ geo, const double* __restrict__ r, const double* __restrict__ minv,
                double* __restrict__ x, double* __restrict__ p, CgScalars* __restrict__ st,
                double* __restrict__ partials, int* __restrict__ err) {
   using S = SliceShape<NP>;
@@ -552,10 +553,11 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, OTF && NP != 6 ? 3 :
   extern __shared__ __align__(128) unsigned char smem[];
   int2* sG = reinterpret_cast<int2*>(smem);
   uint32_t* sD = reinterpret_cast<uint32_t*>(smem + S::kOffD);  // FP16 pairs
+  double* abc = reinterpret_cast<double*>(smem + S::kOffD);     // elements_fp64, in place of sD and sX
   long long* sX = reinterpret_cast<long long*>(smem + S::kOffX);
   uint4* sA = reinterpret_cast<uint4*>(smem + S::kOffA);
   uint2* sB = reinterpret_cast<uint2*>(smem + S::kOffB);
-  unsigned* sMax = reinterpret_cast<unsigned*>(smem + S::kOffM);  // of |u|; of ur and us; of ut
+  unsigned* sMax = reinterpret_cast<unsigned*>(smem + S::kOffM);  // of |u| (near_word); of ur and us; of ut
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + S::kOffBar);
   __shared__ double sRed[32];
 
@@ -694,17 +696,26 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, OTF && NP != 6 ? 3 :
     for (int t = 0; t < 2; ++t)
 #pragma unroll
       for (int x = 0; x < 2; ++x) mh = max(mh, static_cast<unsigned>(__double2hiint(v[t][x])) & 0x7fffffffu);
+    const unsigned top = mh;
     if constexpr (S::kSub == 1)
-      mh = __reduce_max_sync(0xffffffffu, mh);
+      mh = near_word(top, __reduce_max_sync(0xffffffffu, mh), 0xffffffffu);
     else
-      mh = over_element(mh, by_max);
+      mh = near_word(top, over_element(mh, by_max), 0x3333u << (lane & 18));
     put(0, own, mh);
     __syncthreads();
-    mh = 0;
-#pragma unroll
-    for (int q = 0; q < S::kSlots; ++q) mh = max(mh, get(0, q));
-    int emax = static_cast<int>(mh >> 20);
-    bool general = emax == 2047 || abs(1080 - emax + sg) > 700;
+    int emax;
+    unsigned n;  // threads that count
+    if constexpr (S::kSub == 1) {
+      const unsigned all = lane < S::kSlots ? sMax[lane] : 0u;
+      emax = static_cast<int>(__reduce_max_sync(0xffffffffu, all) >> 20);
+      n = __reduce_add_sync(0xffffffffu, static_cast<int>(all >> 20) + kNearWarp >= emax ? all & 63u : 0u);
+    } else {
+      const unsigned m0 = get(0, 0), m1 = get(0, 1);
+      emax = static_cast<int>(by_max(m0, m1) >> 20);
+      n = (static_cast<int>(m0 >> 20) + kNearWarp >= emax ? m0 & 63u : 0u) +
+          (static_cast<int>(m1 >> 20) + kNearWarp >= emax ? m1 & 63u : 0u);
+    }
+    bool general = emax == 2047 || abs(1080 - emax + sg) > 700 || n < S::kFew;
     if (emax < 64) {  // zero, or too small for fixed point
       general = v[0][0] != 0.0 || v[0][1] != 0.0 || v[1][0] != 0.0 || v[1][1] != 0.0;
       emax = 1080;
@@ -784,6 +795,12 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, OTF && NP != 6 ? 3 :
       else
         m = over_element(m, by_or);
       put(1, own, m);
+    } else {  // u over the digits and the exchange
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+          if (in[t][x]) abc[own * P + t * NP2 + off + x] = v[t][x];
     }
     bool ok = true;
     if constexpr (!OTF) ok = mbar_wait_bounded(bar, parity);  // this group's factors
@@ -897,20 +914,17 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, OTF && NP != 6 ? 3 :
         wv[t][1] = to_double(sum[t][1] + r.y, scale);
       }
     } else {
-      double* scratch = reinterpret_cast<double*>(sG);  // the copy has landed; G is read from memory
-      double* res = scratch + 3 * P;
-      for (int q = 0; q < S::kElems && e0 + q < E; ++q) {
-        const double* src = (CG ? p : u) + (e0 + q) * P;
-        if constexpr (OTF)
-          element_fp64<NP>(tab, src, OtfFactors<NP>{tab, coef + (e0 + q) * 24}, scratch, res + q * P);
-        else
-          element_fp64<NP>(tab, src, StoredFactors<NP>{G + (e0 + q) * 6 * P, __ldg(gexp + e0 + q)}, scratch, res + q * P);
-      }
+      elements_fp64<NP, S::kElems>(tab, sG, OTF ? &geo[e0].sg : gexp + e0, OTF ? static_cast<int>(sizeof(GeoElement) / 4) : 1,
+                                   static_cast<int>(group_size(grp)), abc);
 #pragma unroll
       for (int t = 0; t < 2; ++t)
 #pragma unroll
-        for (int x = 0; x < 2; ++x) wv[t][x] = in[t][x] ? res[own * P + t * NP2 + off + x] : 0.0;
+        for (int x = 0; x < 2; ++x) {
+          const double* s = abc + own * P + t * NP2 + off + x;
+          wv[t][x] = in[t][x] ? s[0] + s[S::kElems * P] + s[2 * S::kElems * P] : 0.0;
+        }
       __syncthreads();
+      for (int q = threadIdx.x; q < kSlices * S::kDigit / 2; q += S::kThreads) sD[q] = 0u;  // beyond the points, as at the start
       if (!OTF && threadIdx.x == 0 && more) load_factors(grp + gridDim.x);
     }
     if constexpr (CG) {
@@ -953,7 +967,7 @@ sem_status launch_slice_t(int N, const AxLaunch& a, cudaStream_t s) {
   if (a.grid_out) *a.grid_out = grid;
   k_ax_slice<NP, CG, OTF><<<grid, S::kThreads, S::bytes(OTF), s>>>(
       tab, sl, nodes, a.E, static_cast<const double*>(a.u), static_cast<double*>(a.w), static_cast<const int2*>(a.G),
-      a.gexp, static_cast<const double*>(a.coef), a.geo, static_cast<const double*>(a.r), static_cast<const double*>(a.minv), static_cast<double*>(a.x),
+      a.gexp, a.geo, static_cast<const double*>(a.r), static_cast<const double*>(a.minv), static_cast<double*>(a.x),
       static_cast<double*>(a.p), a.st, a.partials, a.err);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());

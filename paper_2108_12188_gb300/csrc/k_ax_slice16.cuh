@@ -28,6 +28,8 @@ struct Slice16Shape {
   static constexpr size_t kOffM = kOffT + 2 * kSlices * 32 * 16;  // maxima [2][NP]
   static constexpr size_t kOffBar = kOffM + (2 * NP * 4 + 7) / 8 * 8;
   static constexpr size_t kOffTab = (kOffBar + 8 + 15) / 16 * 16;  // on the fly: row tables
+  static constexpr int kFew = kThreads / 4;  // every thread holds points, see kNear
+  static_assert(kSlices * kDigit >= 24 * NP * NP * NP, "the digits' buffer holds the arrays of elements_fp64");
   using Geometry = OtfGeometry<NP, 1, kThreads>;
   static constexpr size_t bytes(bool otf) { return otf ? kOffTab + sizeof(typename Geometry::Tables) : kOffBar + 8; }
 };
@@ -115,13 +117,14 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
     k_ax_slice16(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab<NP> sl,
                  const __grid_constant__ GeoNodes<NP> nodes, int64_t E, const double* __restrict__ u,
                  double* __restrict__ w, const int2* __restrict__ G, const int* __restrict__ gexp,
-                 const double* __restrict__ coef, const GeoElement* __restrict__ geo, const double* __restrict__ r, const double* __restrict__ minv,
+                 const GeoElement* __restrict__ geo, const double* __restrict__ r, const double* __restrict__ minv,
                  double* __restrict__ x, double* __restrict__ p, CgScalars* __restrict__ st,
                  double* __restrict__ partials, int* __restrict__ err) {
   using S = Slice16Shape<NP>;
   constexpr int NP2 = NP * NP, P = NP2 * NP, kMg = magic_groups(NP);
   extern __shared__ __align__(128) unsigned char smem[];
   int2* sG = reinterpret_cast<int2*>(smem);
+  double* abc = reinterpret_cast<double*>(smem + S::kOffD);  // elements_fp64, in place of the digits
   long long* sX = reinterpret_cast<long long*>(smem + S::kOffX);
   uint4* sT = reinterpret_cast<uint4*>(smem + S::kOffT);
   unsigned* sMax = reinterpret_cast<unsigned*>(smem + S::kOffM);
@@ -267,16 +270,15 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
           mh = max(mh, static_cast<unsigned>(__double2hiint(v[a][b][y])) & 0x7fffffffu);
           nonzero |= v[a][b][y] != 0.0;
         }
-    mh = __reduce_max_sync(0xffffffffu, mh);
+    mh = near_word(mh, __reduce_max_sync(0xffffffffu, mh), 0xffffffffu);
     if (lane == 0) sMax[warp] = mh;
     __syncthreads();
-    mh = 0;
-#pragma unroll
-    for (int q = 0; q < NP; ++q) mh = max(mh, sMax[q]);
-    int emax = static_cast<int>(mh >> 20);
-    bool general = emax == 2047 || abs(1080 - emax + sg) > 700;
+    const unsigned all = lane < NP ? sMax[lane] : 0u;
+    int emax = static_cast<int>(__reduce_max_sync(0xffffffffu, all) >> 20);
+    const bool near = static_cast<int>(all >> 20) + kNearWarp >= emax;
+    bool slow = emax == 2047 || abs(1080 - emax + sg) > 700 || __reduce_add_sync(0xffffffffu, near ? all & 63u : 0u) < S::kFew;
     if (emax < 64) {  // zero, or too small for fixed point
-      general = nonzero;
+      slow = __syncthreads_or(nonzero);
       emax = 1080;
     }
     if (threadIdx.x == 0 && more) {  // the next element's vectors into L2
@@ -302,7 +304,7 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
         put_digits(a, b, d);
       }
     if constexpr (OTF) S::Geometry::columns(tables, geo, e, 1, sG);
-    const bool slow = __syncthreads_or(general);
+    __syncthreads();
 
     // phase 1
     long long vr[2][2][2], vs[2][2][2];
@@ -347,6 +349,14 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
           for (int y = 0; y < 2; ++y) m |= magnitude(vr[a][b][y]) | magnitude(vs[a][b][y]);
       m = __reduce_or_sync(0xffffffffu, m);
       if (lane == 0) sMax[NP + warp] = m;
+    } else {  // u over the digits
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+          for (int y = 0; y < 2; ++y)
+            if (in(a, b, y)) abc[warp * NP2 + off(a, b) + y] = v[a][b][y];
     }
     bool ok = true;
     if constexpr (!OTF) ok = mbar_wait_bounded(bar, parity);  // this element's factors
@@ -463,19 +473,19 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
           wv[a][b][1] = to_double(sum[a][b][1] + t.y, scale);
         }
     } else {
-      double* scratch = reinterpret_cast<double*>(sG);  // the copy has landed; G is read from memory
-      double* res = scratch + 3 * P;
-      if constexpr (OTF)
-        element_fp64<NP>(tab, (CG ? p : u) + e * P, OtfFactors<NP>{tab, coef + e * 24}, scratch, res);
-      else
-        element_fp64<NP>(tab, (CG ? p : u) + e * P, StoredFactors<NP>{G + e * 6 * P, sg}, scratch, res);
+      elements_fp64<NP, 1>(tab, sG, OTF ? &geo[e].sg : gexp + e, 0, 1, abc);
 #pragma unroll
       for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int b = 0; b < 2; ++b)
 #pragma unroll
-          for (int y = 0; y < 2; ++y) wv[a][b][y] = in(a, b, y) ? res[warp * NP2 + off(a, b) + y] : 0.0;
+          for (int y = 0; y < 2; ++y) {
+            const double* s = abc + warp * NP2 + off(a, b) + y;
+            wv[a][b][y] = in(a, b, y) ? s[0] + s[P] + s[2 * P] : 0.0;
+          }
       __syncthreads();
+      for (unsigned q = threadIdx.x; q < kSlices * S::kDigit / 4; q += S::kThreads)  // beyond the points, as at the start
+        reinterpret_cast<uint32_t*>(smem + S::kOffD)[q] = 0u;
       if (!OTF && threadIdx.x == 0 && more) load_factors(e + gridDim.x);
     }
 #pragma unroll
@@ -519,7 +529,7 @@ sem_status launch_slice16_t(int N, const AxLaunch& a, cudaStream_t s) {
   if (a.grid_out) *a.grid_out = grid;
   k_ax_slice16<NP, CG, OTF><<<grid, S::kThreads, S::bytes(OTF), s>>>(
       tab, sl, nodes, a.E, static_cast<const double*>(a.u), static_cast<double*>(a.w), static_cast<const int2*>(a.G),
-      a.gexp, static_cast<const double*>(a.coef), a.geo, static_cast<const double*>(a.r), static_cast<const double*>(a.minv), static_cast<double*>(a.x),
+      a.gexp, a.geo, static_cast<const double*>(a.r), static_cast<const double*>(a.minv), static_cast<double*>(a.x),
       static_cast<double*>(a.p), a.st, a.partials, a.err);
   count_launch();
   SEM_CUDA_TRY(cudaGetLastError());
