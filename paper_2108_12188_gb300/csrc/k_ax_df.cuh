@@ -312,7 +312,7 @@ struct FixedScale {
   __device__ __forceinline__ void init(int sg) {
     s32 = pow2f(32 - sg);
     s16 = pow2f(16 - sg);
-    s0 = pow2f(-sg);
+    s0 = sg < kSgFinite ? __int_as_float(0x7fc00000) : pow2f(-sg);
   }
   // X = (hi & ~7) 2^32 + ((hi & 7) 2^16 + lo >> 16) 2^16 + (lo & 0xffff), three exact floats (|hi| <= 2^27),
   // added into a pair: 48 bits of the value itself

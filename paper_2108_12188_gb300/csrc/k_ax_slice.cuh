@@ -388,7 +388,10 @@ __device__ __noinline__ void elements_fp64(const GllParam<NP, double>& tab, cons
       const int2 x = G[(el * 6 + m) * P + r];
       const long long v = static_cast<long long>(x.y) * 4294967296ll + x.x;
       const int k = -(e + c[m < 3 ? 0 : m < 5 ? 1 : 2] + c[m < 3 ? m : m < 5 ? m - 2 : 2]);
-      g[m] = abs(e) < 900 ? to_double(v, k) : scalbn(static_cast<double>(v), k);  // (to_double wants a normal result)
+      // (to_double wants a normal result)
+      g[m] = abs(e) < 900    ? to_double(v, k)
+             : e > kSgFinite ? scalbn(static_cast<double>(v), k)
+                             : __hiloint2double(0x7ff80000, 0);
     }
     const double ur = B[q], us = A[q], ut = C[q];
     B[q] = g[0] * ur + g[1] * us + g[2] * ut;
@@ -717,7 +720,7 @@ __global__ void __launch_bounds__(SliceShape<NP>::kThreads, OTF && NP != 6 ? 3 :
     }
     bool general = emax == 2047 || abs(1080 - emax + sg) > 700 || n < S::kFew;
     if (emax < 64) {  // zero, or too small for fixed point
-      general = v[0][0] != 0.0 || v[0][1] != 0.0 || v[1][0] != 0.0 || v[1][1] != 0.0;
+      general = v[0][0] != 0.0 || v[0][1] != 0.0 || v[1][0] != 0.0 || v[1][1] != 0.0 || sg < kSgFinite;
       emax = 1080;
     }
     if (threadIdx.x == 0 && more) {  // the next group's vectors into L2

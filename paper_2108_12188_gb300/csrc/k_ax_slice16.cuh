@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(Slice16Shape<NP>::kThreads, 1)
     const bool near = static_cast<int>(all >> 20) + kNearWarp >= emax;
     bool slow = emax == 2047 || abs(1080 - emax + sg) > 700 || __reduce_add_sync(0xffffffffu, near ? all & 63u : 0u) < S::kFew;
     if (emax < 64) {  // zero, or too small for fixed point
-      slow = __syncthreads_or(nonzero);
+      slow = __syncthreads_or(nonzero || sg < kSgFinite);
       emax = 1080;
     }
     if (threadIdx.x == 0 && more) {  // the next element's vectors into L2

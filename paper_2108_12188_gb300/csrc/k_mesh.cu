@@ -167,9 +167,9 @@ __global__ void k_fixed_factors(const __grid_constant__ GllAll tab, int Np, int 
   if (threadIdx.x == 0) sMin = 4000;
   __syncthreads();
   int most[5] = {-4000, -4000, -4000, -4000, -4000}, least = 4000;
-  auto exponent = [](double v) {
+  auto exponent = [](double v) {  // (4000: no finite number, see kSgFinite)
     const int ex = (__double2hiint(v) >> 20) & 0x7ff;
-    return ex == 0 || ex == 0x7ff ? -4000 : ex - 1022;
+    return ex == 0 ? -4000 : ex == 0x7ff ? 4000 : ex - 1022;
   };
   // of a bound that rounding may have put below a power of two it reaches: the high word one up
   auto exponent_up = [&](double v) { return exponent(__hiloint2double(__double2hiint(v) + 1, 0)); };

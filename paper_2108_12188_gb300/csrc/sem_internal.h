@@ -158,6 +158,9 @@ constexpr bool f64x_plain_pairs(int N, int64_t E) { return N == 7 && E < 2560; }
 __host__ __device__ constexpr int fixed_row_scale(int NP, int i) {
   return i == 0 || i == NP - 1 ? (NP <= 4 ? 1 : 2) : 0;
 }
+// An element with an infinite factor (c . c overflows from edges of 1e77) has its exponent sg below this and stands for
+// NaN factors; finite ones have theirs above.
+constexpr int kSgFinite = -1100;
 
 // ---- reduction scratch ----
 constexpr int kRedMax = 8192;  // upper bound of blocks of any reducing launch
