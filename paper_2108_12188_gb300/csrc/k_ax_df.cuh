@@ -302,20 +302,25 @@ struct OtfColumnDf {
   }
 };
 
-// Scales that turn fixed-point factors into float pairs: 2^(32 - sg), 2^(16 - sg), 2^-sg (0 below FP32's
-// normal range).
+// Scales that turn fixed-point factors into float pairs: X 2^-sg = (X 2^(2 half - sg)) 2^-(2 half) with the first in the middle of
+// FP32's range, so that no part of X falls out of it while the factor itself is inside; `half` goes into each of the two row
+// scales that a factor takes (below 2^-149 together: 0, above 2^127: infinity).
 struct FixedScale {
   float s32, s16, s0;
+  int half;
   __device__ __forceinline__ static float pow2f(int e) {
-    return e < -126 ? 0.f : __int_as_float((127 + min(e, 127)) << 23);
+    return e < -126 ? 0.f : __int_as_float((e > 127 ? 255 : 127 + e) << 23);
   }
   __device__ __forceinline__ void init(int sg) {
-    s32 = pow2f(32 - sg);
-    s16 = pow2f(16 - sg);
-    s0 = sg < kSgFinite ? __int_as_float(0x7fc00000) : pow2f(-sg);
+    half = (sg - 48) >> 1;
+    const int r = 2 * half - sg;  // -48 or -49
+    s32 = pow2f(32 + r);
+    s16 = pow2f(16 + r);
+    s0 = sg < kSgFinite ? __int_as_float(0x7fc00000) : pow2f(r);
   }
+  __device__ __forceinline__ float row(int c) const { return pow2f(-half - c); }  // c: fixed_row_scale
   // X = (hi & ~7) 2^32 + ((hi & 7) 2^16 + lo >> 16) 2^16 + (lo & 0xffff), three exact floats (|hi| <= 2^27),
-  // added into a pair: 48 bits of the value itself
+  // added into a pair: 48 bits of the value itself. f: the product of its two row()
   __device__ __forceinline__ df2 pair(int2 x, float f) const {
     const float a = static_cast<float>(x.y & ~7) * s32;
     const float b = static_cast<float>(((x.y & 7) << 16) + (x.x >> 16)) * s16;
@@ -533,8 +538,8 @@ __global__ void __launch_bounds__(NP * NP * ax_epb<NP>(), MINB)
       float fi = 1.f, fj = 1.f;
       if constexpr (GK == kGkFixed) {
         fx.init(valid ? __ldg(gexp + e) : 0);
-        fi = FixedScale::pow2f(-fixed_row_scale(NP, i));
-        fj = FixedScale::pow2f(-fixed_row_scale(NP, j));
+        fi = fx.row(fixed_row_scale(NP, i));
+        fj = fx.row(fixed_row_scale(NP, j));
       }
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
@@ -545,7 +550,7 @@ __global__ void __launch_bounds__(NP * NP * ax_epb<NP>(), MINB)
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
         df2 g[6];
-        const float fk = GK == kGkFixed ? FixedScale::pow2f(-fixed_row_scale(NP, k)) : 1.f;
+        const float fk = GK == kGkFixed ? fx.row(fixed_row_scale(NP, k)) : 1.f;
 #pragma unroll
         for (int m = 0; m < 6; ++m) {
           const double* src = (GST != 6 * P && m >= 3) ? gH : gE;
