@@ -230,6 +230,46 @@ sem_status launch_ax_any(sem_mesh m, sem_prec prec, sem_ax_variant v, bool cg, A
   return prec == SEM_F64 ? launch_ax_f64(m->N, v, cg, a, s) : launch_ax_f32(m->N, v, cg, a, s);
 }
 
+FactorArrays factor_arrays(int N, int64_t E, unsigned flags) {
+  const bool f64 = flags & SEM_MESH_F64_STORED, f64x = flags & SEM_MESH_F64X_STORED;
+  const size_t e = static_cast<size_t>(E), P = static_cast<size_t>(N + 1) * (N + 1) * (N + 1);
+  FactorArrays a{};
+  a.g64 = f64 && !ax_slice_order(N);
+  a.fixed = (f64 && ax_slice_order(N)) || (f64x && f64x_on_slices(N));
+  a.geo = ax_slice_order(N);
+  a.pairs = f64x && (!f64x_on_slices(N) || f64x_plain_pairs(N, E));
+  a.g32 = flags & SEM_MESH_F32_STORED;
+  a.scale = flags & SEM_MESH_OTF_SCALE;
+  a.bytes = e * ((a.g64 ? 48 * P : 0) + (a.fixed ? 48 * P + 4 : 0) + (a.geo ? sizeof(GeoElement) : 0) + (a.pairs ? 48 * P : 0) +
+                 (a.g32 ? 4 * static_cast<size_t>(factor_stride(N + 1, true)) : 0) + (a.scale ? 12 * P : 0));
+  return a;
+}
+
+bool small_cg_mesh(int64_t E) { return E < host_sm_count(); }
+
+// FP64 factors for the persistent small-mesh CG where the mesh holds them in fixed point only; once per mesh.
+sem_status ensure_small_factors(sem_mesh m, cudaStream_t s) {
+  if (m->G64) return SEM_OK;
+  note_stream(m, s);
+  const size_t count = static_cast<size_t>(m->E) * 6 * m->Np * m->Np * m->Np;
+  size_t bytes = 0;
+  int* bad = nullptr;
+  SEM_TRY(dmalloc(&bad, 1, nullptr, s));
+  sem_status st = dmalloc(&m->G64, count, &bytes, s);
+  if (st == SEM_OK)
+    st = launch_geometry(m->N, m->E, m->coef64, m->G64, nullptr, nullptr, nullptr, bad, factor_stride(m->Np, false),
+                         factor_stride(m->Np, true), s);
+  dfree(bad, s);
+  const cudaError_t e = cudaStreamSynchronize(s);
+  if (st == SEM_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize (FP64 factors)");
+  if (st != SEM_OK) {
+    dfree(m->G64, s);
+    return st;
+  }
+  m->device_bytes += bytes;
+  return SEM_OK;
+}
+
 // Jacobi inverse diagonal, built once per mesh in FP64 (and rounded to FP32).
 sem_status ensure_jacobi(sem_mesh m, cudaStream_t s) {
   if (m->minv64) return SEM_OK;
@@ -367,20 +407,16 @@ extern "C" sem_status sem_mesh_create(int N, int64_t nv, const double* vert_xyz,
     SEM_STEP(dmalloc(&bad, 1, nullptr, s));
     SEM_STEP(dmalloc(&m->coef64, static_cast<size_t>(E) * 24, &acc, s));
     SEM_STEP(dmalloc(&m->coef32, static_cast<size_t>(E) * 24, &acc, s));
-    // (the persistent CG kernel of small meshes, use_graph = 2, reads FP64 factors at every order)
-    if ((flags & SEM_MESH_F64_STORED) && (!ax_slice_order(N) || E < host_sm_count()))
-      SEM_STEP(dmalloc(&m->G64, static_cast<size_t>(E * 6 * P), &acc, s));
-    const bool x_fixed = (flags & SEM_MESH_F64X_STORED) && f64x_on_slices(N);
-    if (((flags & SEM_MESH_F64_STORED) && ax_slice_order(N)) || x_fixed) {
+    const FactorArrays arrays = factor_arrays(N, E, flags);
+    if (arrays.g64) SEM_STEP(dmalloc(&m->G64, static_cast<size_t>(E * 6 * P), &acc, s));
+    if (arrays.fixed) {
       SEM_STEP(dmalloc(&m->GI, static_cast<size_t>(E * 6 * P), &acc, s));
       SEM_STEP(dmalloc(&m->gexp, static_cast<size_t>(E), &acc, s));
     }
-    if (ax_slice_order(N)) SEM_STEP(dmalloc(&m->geo, static_cast<size_t>(E), &acc, s));
-    if ((flags & SEM_MESH_F64X_STORED) && (!x_fixed || f64x_plain_pairs(N, E)))
-      SEM_STEP(dmalloc(&m->Gx, static_cast<size_t>(2 * E * 6 * P), &acc, s));
-    if (flags & SEM_MESH_F32_STORED)
-      SEM_STEP(dmalloc(&m->G32, static_cast<size_t>(E * factor_stride(m->Np, true)), &acc, s));
-    if (flags & SEM_MESH_OTF_SCALE) {
+    if (arrays.geo) SEM_STEP(dmalloc(&m->geo, static_cast<size_t>(E), &acc, s));
+    if (arrays.pairs) SEM_STEP(dmalloc(&m->Gx, static_cast<size_t>(2 * E * 6 * P), &acc, s));
+    if (arrays.g32) SEM_STEP(dmalloc(&m->G32, static_cast<size_t>(E * factor_stride(m->Np, true)), &acc, s));
+    if (arrays.scale) {
       SEM_STEP(dmalloc(&m->scale64, static_cast<size_t>(E * P), &acc, s));
       SEM_STEP(dmalloc(&m->scale32, static_cast<size_t>(E * P), &acc, s));
     }
@@ -778,6 +814,8 @@ sem_status cg_alloc(sem_mesh m, sem_prec prec, sem_ax_variant v, int precond, do
   if (v == SEM_AX_OTF_SCALE && !has_scales(m))
     return fail(SEM_ERR_ARG, "per-point scales were not requested at mesh creation (SEM_MESH_OTF_SCALE)");
   if (cg_layout(prec)) SEM_TRY(ensure_cg_layout(m, m->home));
+  if (use_graph == 2 && prec == SEM_F64 && v == SEM_AX_STORED && small_cg_mesh(m->E))
+    SEM_TRY(ensure_small_factors(m, m->home));
   sem_cg c = new sem_cg_s();
   c->m = m;
   c->prec = prec;
@@ -919,7 +957,7 @@ sem_status cg_enqueue_iteration(sem_cg c, cudaStream_t s) {
 // use_graph = 2: FP64 CG with stored factors on a mesh with fewer elements than the device has
 // SMs runs in the persistent kernel (k_cg_small.cu), a run of iterations per launch.
 bool small_path(sem_cg c) {
-  if (c->use_graph != 2 || c->prec != SEM_F64 || !c->m->G64 || c->m->E >= host_sm_count()) return false;
+  if (c->use_graph != 2 || c->prec != SEM_F64 || !c->m->G64 || !small_cg_mesh(c->m->E)) return false;
   sem_ax_variant v;
   int shape;
   resolve_variant(c->m, SEM_F64, c->variant, &v, &shape);

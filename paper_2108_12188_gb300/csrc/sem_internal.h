@@ -162,6 +162,16 @@ __host__ __device__ constexpr int fixed_row_scale(int NP, int i) {
 // NaN factors; finite ones have theirs above.
 constexpr int kSgFinite = -1100;
 
+// Arrays of geometric factors that a mesh holds for its flags, and their device bytes (api.cpp). At the orders of
+// ax_slice_order the FP64 values of the persistent small-mesh CG are made by the first solver that takes it.
+struct FactorArrays {
+  bool g64, fixed, geo, pairs, g32, scale;
+  size_t bytes;
+};
+FactorArrays factor_arrays(int N, int64_t E, unsigned flags);
+// The FP64 CG on this mesh would run in the persistent kernel (use_graph = 2).
+bool small_cg_mesh(int64_t E);
+
 // ---- reduction scratch ----
 constexpr int kRedMax = 8192;  // upper bound of blocks of any reducing launch
 
@@ -251,7 +261,7 @@ struct sem_mesh_s {
   // device arrays
   double* coef64 = nullptr;   // [E][24] trilinear coefficients a0..a7 (x, y, z)
   float* coef32 = nullptr;    // [E][24] rounded to FP32
-  double* G64 = nullptr;      // [E][6][P] or null (ax_slice_order: only for fewer elements than SMs)
+  double* G64 = nullptr;      // [E][6][P] or null (ax_slice_order: once a solver has taken use_graph = 2)
   int2* GI = nullptr;         // [E][6][P] fixed-point factors (ax_slice_order; at N = 7 for SEM_F64X too) or null
   int* gexp = nullptr;        // [E] their exponents sg
   sem::GeoElement* geo = nullptr;  // [E] elements for factors rebuilt in fixed point (ax_slice_order), or null: not this mesh

@@ -85,19 +85,38 @@ struct sem_server_s {
 
 namespace {
 
-// Device bytes of one request: mesh (coefficients, segments, multiplicities), stored factors
-// if the options need them, Jacobi inverse (FP64 + FP32), right-hand side and solution,
-// FP64 CG or refinement work vectors plus the FP32 inner CG.
-size_t estimate_bytes(int64_t E, int N, const sem_cg_opts& o) {
-  const size_t Np = static_cast<size_t>(N) + 1;
-  const size_t n = static_cast<size_t>(E) * Np * Np * Np;
-  size_t b = static_cast<size_t>(E) * 24 * 12 + 5 * n + 12 * n + 16 * n;
-  const bool f64_stored = o.variant == SEM_AX_STORED;
-  const bool f32_stored = o.mixed && o.inner_variant == SEM_AX_STORED;
-  if (f64_stored) b += 48 * n;
-  if (f32_stored) b += 24 * n;
-  b += o.mixed ? (16 * n + 8 * n + 16 * n) : 32 * n;
+// Flags of a request's mesh: the stored factors its options read. (Where SEM_F64X runs on the FP64 operator's
+// factors, CG reads no others; the refinement's residuals may take the float pairs.)
+unsigned request_flags(int N, const sem_cg_opts& o) {
+  unsigned flags = 0;
+  if (o.variant == SEM_AX_STORED)
+    flags |= o.f64_arith && (o.mixed || !sem::f64x_on_slices(N)) ? SEM_MESH_F64X_STORED : SEM_MESH_F64_STORED;
+  if (o.mixed && o.inner_variant == SEM_AX_STORED) flags |= SEM_MESH_F32_STORED;
+  return flags;
+}
+
+// Gather-scatter records: 4 bytes of index for every point on an element's boundary, at most 2 of padding and mask.
+size_t segment_bytes(int64_t E, int N) {
+  const size_t Np = static_cast<size_t>(N) + 1, inner = N > 1 ? (Np - 2) * (Np - 2) * (Np - 2) : 0;
+  return 6 * static_cast<size_t>(E) * (Np * Np * Np - inner);
+}
+
+// Device bytes of a solve beside its mesh: right-hand side and solution, Jacobi inverse (FP64 + FP32), and FP64 CG (with
+// the segments in its layout, and FP64 factors for the persistent kernel) or refinement work vectors plus the FP32
+// inner CG.
+size_t solve_bytes(int64_t E, int N, const sem_cg_opts& o) {
+  const size_t Np = static_cast<size_t>(N) + 1, n = static_cast<size_t>(E) * Np * Np * Np;
+  size_t b = 16 * n + 12 * n + (o.mixed ? 16 * n + 8 * n + 16 * n : 32 * n + segment_bytes(E, N));
+  if (!o.mixed && !o.f64_arith && o.use_graph == 2 && o.variant == SEM_AX_STORED && sem::ax_slice_order(N) &&
+      sem::small_cg_mesh(E))
+    b += 48 * n;
   return b + (8u << 20);
+}
+
+// Device bytes of one request: mesh (coefficients, segments, multiplicities, factors) and solve.
+size_t estimate_bytes(int64_t E, int N, const sem_cg_opts& o) {
+  const size_t Np = static_cast<size_t>(N) + 1, e = static_cast<size_t>(E), n = e * Np * Np * Np;
+  return e * 24 * 12 + n + segment_bytes(E, N) + sem::factor_arrays(N, E, request_flags(N, o)).bytes + solve_bytes(E, N, o);
 }
 
 // CUDA stream priority of a request's work: with size priorities, the fewer local points the
@@ -123,9 +142,7 @@ void run_request(sem_server srv, Request* r) {
   const double t0 = now_ms();
   if (cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, request_priority(srv, r->n_local)) != cudaSuccess)
     st = SEM_ERR_CUDA;
-  unsigned flags = 0;
-  if (r->opts.variant == SEM_AX_STORED) flags |= r->opts.f64_arith ? SEM_MESH_F64X_STORED : SEM_MESH_F64_STORED;
-  if (r->opts.mixed && r->opts.inner_variant == SEM_AX_STORED) flags |= SEM_MESH_F32_STORED;
+  const unsigned flags = request_flags(r->N, r->opts);
   if (r->mesh) {  // prebuilt mesh: now the server's
     mesh = r->mesh;
     r->mesh = nullptr;
@@ -464,10 +481,7 @@ extern "C" sem_status sem_server_submit_mesh(sem_server srv, sem_mesh mesh, cons
     r->n_local = mesh->n;
     r->b_host.assign(b_host, b_host + mesh->n);
     r->opts = *opts;
-    // the mesh's memory plus the solver's: b, x, the Jacobi inverse (FP64 and FP32) and the
-    // CG work vectors (FP64 CG, or FP32 CG with the FP64 refinement buffers)
-    const size_t n = static_cast<size_t>(mesh->n);
-    r->est_bytes = mesh->device_bytes + 16 * n + 12 * n + (opts->mixed ? 40 * n : 32 * n) + (8u << 20);
+    r->est_bytes = mesh->device_bytes + solve_bytes(mesh->E, mesh->N, *opts);
     r->batched = routes_to_batch(srv, r->n_local, r->opts);
     if (r->est_bytes > srv->budget) return fail(SEM_ERR_ARG, "request needs more device memory than the budget");
     // the caller's streams may go away: finish their work on the mesh now (without the lock)
