@@ -238,14 +238,15 @@ sem_status sem_rhs_sine(sem_mesh mesh, int a, int b, int c, sem_prec prec, void*
  * or on-the-fly with per-point scale where available, times two block shapes: elements per
  * thread block; the per-point-scale variant has one shape; for FP32 on the fly at N = 7 also
  * shape 3, the line contractions on the tensor cores: mma.sync TF32 with split operands;
- * for SEM_F64X stored and on the fly, one shape each) with CUDA events over `reps` launches each, and records the fastest for the mesh's order
- * and the precision, process-wide; SEM_AX_AUTO then uses it, and explicit variants use the
- * faster block shape. Synchronises `stream`. sem_autotune_save / sem_autotune_load write and
+ * for SEM_F64X stored and on the fly and for SEM_F64 on the tensor cores, one shape each) with CUDA events over `reps` launches
+ * each, and records the fastest for the mesh's order, the precision and the kernels the mesh runs (SEM_F64 on the fly: on the tensor
+ * cores or not; SEM_F64X at order 7: float pairs or not), process-wide; SEM_AX_AUTO then uses it, and explicit variants that were
+ * timed use the faster block shape. Synchronises `stream`. sem_autotune_save / sem_autotune_load write and
  * read the table as text, keyed by the GPU name (a table from another GPU model is refused
  * with SEM_ERR_ARG). The paper has no tuner (its kernels are fixed FPGA pipelines). */
 typedef struct {
   int variant;            /* sem_ax_variant */
-  int shape;              /* block shape choice 0 / 1, or 3 (tensor cores) */
+  int shape;              /* block shape choice 0 / 1, or 3 (FP32 on the tensor cores) */
   int elements_per_block;
   double ms;              /* mean time of one A_L application */
 } sem_tune_entry;

@@ -156,17 +156,27 @@ void free_mesh(sem_mesh m) {
   m->used.clear();
 }
 
-// Process-wide tuning results per precision (F64, F32, F64X) and order: the best variant and,
-// for each variant, its faster block shape.
+// Process-wide tuning results per precision (F64, F32, F64X), order and kind of mesh: the best variant and, for each
+// variant, its faster block shape (kUntunedShape where none was timed or set).
 struct TuneSlot {
   bool valid = false;
   sem_ax_variant best = SEM_AX_STORED;
-  int shape[3] = {0, 0, 0};  // per variant slot: STORED, OTF, OTF_SCALE
+  int shape[3] = {kUntunedShape, kUntunedShape, kUntunedShape};  // per variant slot: STORED, OTF, OTF_SCALE
   double ms[3] = {0, 0, 0};
 };
+// Meshes of one order whose operators are not the same kernels: SEM_F64 on the fly rebuilds factors in fixed point
+// or in FP64 (geo), SEM_F64X at order 7 has float pairs or not.
+constexpr int kTuneKinds = 2;
+int tune_kind(sem_mesh m, sem_prec prec) {
+  return prec == SEM_F64 ? m->geo != nullptr : prec == SEM_F64X ? f64x_on_slices(m->N) && m->Gx != nullptr : 0;
+}
+// The operator has no block shapes to choose from: the tensor-core kernels of SEM_F64.
+bool ax_one_shape(sem_mesh m, sem_prec prec, sem_ax_variant v) {
+  return prec == SEM_F64 && (v == SEM_AX_STORED ? ax_slice_order(m->N) : m->geo != nullptr);
+}
 inline int vslot(sem_ax_variant v) { return v == SEM_AX_OTF_SCALE ? 2 : static_cast<int>(v); }
 std::mutex g_tune_mu;
-TuneSlot g_tune[3][SEM_MAX_N + 1];
+TuneSlot g_tune[3][kTuneKinds][SEM_MAX_N + 1];
 
 // Stored factors the local operator of precision `prec` reads: FP32 for SEM_F32; for SEM_F64X the
 // float pairs if the mesh has them, else the FP64 operator's (split in the kernel); those are FP64 values,
@@ -191,7 +201,7 @@ bool has_scales(sem_mesh m) { return m->scale64 != nullptr; }
 // Resolves SEM_AX_AUTO and picks the tuned block shape.
 void resolve_variant(sem_mesh m, sem_prec prec, sem_ax_variant v, sem_ax_variant* out_v, int* out_shape) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
-  const TuneSlot& t = g_tune[prec][m->N];
+  const TuneSlot& t = g_tune[prec][tune_kind(m, prec)][m->N];
   sem_ax_variant r = v;
   if (v == SEM_AX_AUTO) {
     if (t.valid && (t.best == SEM_AX_OTF || (t.best == SEM_AX_STORED && has_factors(m, prec)) ||
@@ -202,7 +212,7 @@ void resolve_variant(sem_mesh m, sem_prec prec, sem_ax_variant v, sem_ax_variant
     if (prec == SEM_F64X && r == SEM_AX_OTF_SCALE) r = has_factors(m, prec) ? SEM_AX_STORED : SEM_AX_OTF;
   }
   *out_v = r;
-  *out_shape = t.valid ? t.shape[vslot(r)] : kUntunedShape;
+  *out_shape = t.shape[vslot(r)];
 }
 
 }  // namespace
@@ -1406,7 +1416,8 @@ extern "C" sem_status sem_autotune(sem_mesh m, sem_prec prec, int reps, sem_tune
       if (v == SEM_AX_OTF_SCALE && !has_scales(m)) continue;
       for (int shape : {0, 1, kTensorShape}) {
         if (st != SEM_OK) break;
-        if (shape == 1 && (prec == SEM_F64X || v == SEM_AX_OTF_SCALE ||
+        const bool one_shape = ax_one_shape(m, prec, v);
+        if (shape == 1 && (prec == SEM_F64X || v == SEM_AX_OTF_SCALE || one_shape ||
                            ax_elements_per_block(m->N, 1) == ax_elements_per_block(m->N, 0)))
           continue;
         if (shape == kTensorShape && !ax_tensor_available(m->N, prec, v)) continue;
@@ -1437,7 +1448,10 @@ extern "C" sem_status sem_autotune(sem_mesh m, sem_prec prec, int reps, sem_tune
         sem_tune_entry& c = rep->candidates[rep->n_candidates++];
         c.variant = v;
         c.shape = shape;
-        c.elements_per_block = prec == SEM_F64X ? 0 : shape == kTensorShape ? 1 : ax_elements_per_block(m->N, shape);
+        c.elements_per_block = prec == SEM_F64X      ? 0
+                               : shape == kTensorShape ? 1
+                               : one_shape             ? ax_slice_elements(m->N)
+                                                       : ax_elements_per_block(m->N, shape);
         c.ms = ms / reps;
       }
     }
@@ -1457,7 +1471,7 @@ extern "C" sem_status sem_autotune(sem_mesh m, sem_prec prec, int reps, sem_tune
       const int slot = vslot(static_cast<sem_ax_variant>(c.variant));
       if (c.ms < best_v[slot]) {
         best_v[slot] = c.ms;
-        t.shape[slot] = c.shape;
+        t.shape[slot] = ax_one_shape(m, prec, static_cast<sem_ax_variant>(c.variant)) ? kUntunedShape : c.shape;
         t.ms[slot] = c.ms;
       }
       if (c.ms < best) {
@@ -1467,7 +1481,7 @@ extern "C" sem_status sem_autotune(sem_mesh m, sem_prec prec, int reps, sem_tune
       }
     }
     std::lock_guard<std::mutex> lock(g_tune_mu);
-    g_tune[prec][m->N] = t;
+    g_tune[prec][tune_kind(m, prec)][m->N] = t;
     return SEM_OK;
   });
 }
@@ -1482,13 +1496,15 @@ extern "C" sem_status sem_autotune_set(int N, sem_prec prec, sem_ax_variant vari
                     (shape == kTensorShape && ax_tensor_available(N, prec, variant));
     if (!ok) return fail(SEM_ERR_ARG, "block shape choice not available for this order, precision and variant");
     std::lock_guard<std::mutex> lock(g_tune_mu);
-    TuneSlot& t = g_tune[prec][N];
-    if (!t.valid) {
-      t = TuneSlot{};
-      t.valid = true;
-      t.best = variant;
+    for (auto& kind : g_tune[prec]) {
+      TuneSlot& t = kind[N];
+      if (!t.valid) {
+        t = TuneSlot{};
+        t.valid = true;
+        t.best = variant;
+      }
+      t.shape[vslot(variant)] = shape;
     }
-    t.shape[vslot(variant)] = shape;
     return SEM_OK;
   });
 }
@@ -1496,8 +1512,9 @@ extern "C" sem_status sem_autotune_set(int N, sem_prec prec, sem_ax_variant vari
 extern "C" sem_status sem_autotune_clear(void) {
   return guarded([&]() -> sem_status {
     std::lock_guard<std::mutex> lock(g_tune_mu);
-    for (auto& row : g_tune)
-      for (TuneSlot& t : row) t = TuneSlot{};
+    for (auto& prec : g_tune)
+      for (auto& kind : prec)
+        for (TuneSlot& t : kind) t = TuneSlot{};
     return SEM_OK;
   });
 }
@@ -1507,15 +1524,16 @@ extern "C" sem_status sem_autotune_save(const char* path) {
     if (!path) return fail(SEM_ERR_ARG, "null path");
     std::ofstream f(path);
     if (!f) return fail(SEM_ERR_ARG, std::string("cannot write ") + path);
-    f << "sem-autotune 2 " << device_name() << "\n";
+    f << "sem-autotune 3 " << device_name() << "\n";
     std::lock_guard<std::mutex> lock(g_tune_mu);
     for (int p = 0; p < 3; ++p)
-      for (int N = 1; N <= SEM_MAX_N; ++N) {
-        const TuneSlot& t = g_tune[p][N];
-        if (t.valid)
-          f << p << " " << N << " " << t.best << " " << t.shape[0] << " " << t.shape[1] << " " << t.shape[2] << " "
-            << t.ms[0] << " " << t.ms[1] << " " << t.ms[2] << "\n";
-      }
+      for (int kind = 0; kind < kTuneKinds; ++kind)
+        for (int N = 1; N <= SEM_MAX_N; ++N) {
+          const TuneSlot& t = g_tune[p][kind][N];
+          if (t.valid)
+            f << p << " " << N << " " << t.best << " " << t.shape[0] << " " << t.shape[1] << " " << t.shape[2] << " "
+              << t.ms[0] << " " << t.ms[1] << " " << t.ms[2] << " " << kind << "\n";
+        }
     return f ? SEM_OK : fail(SEM_ERR_ARG, "write failed");
   });
 }
@@ -1528,25 +1546,31 @@ extern "C" sem_status sem_autotune_load(const char* path) {
     std::string magic, gpu;
     int version = 0;
     f >> magic >> version >> gpu;
-    if (magic != "sem-autotune" || version != 2) return fail(SEM_ERR_ARG, "not a tuning table");
+    if (magic != "sem-autotune" || (version != 2 && version != 3)) return fail(SEM_ERR_ARG, "not a tuning table");
     if (gpu != device_name()) return fail(SEM_ERR_ARG, "tuning table was made on " + gpu);
-    int p, N, best, s0, s1, s2;
+    // version 2: no kind of mesh (its lines are for every kind), no untuned shapes
+    const int least = version == 2 ? 0 : kUntunedShape;
+    int p, N, best, s0, s1, s2, kind = 0;
     double m0, m1, m2;
     std::lock_guard<std::mutex> lock(g_tune_mu);
-    while (f >> p >> N >> best >> s0 >> s1 >> s2 >> m0 >> m1 >> m2) {
-      if (p < 0 || p > 2 || N < 1 || N > SEM_MAX_N || !(best == 0 || best == 1 || best == 3) || s0 < 0 || s0 > 1 ||
-          !(s1 == 0 || s1 == 1 || (s1 == kTensorShape && ax_tensor_available(N, static_cast<sem_prec>(p), SEM_AX_OTF))) ||
-          s2 != 0)
+    while (f >> p >> N >> best >> s0 >> s1 >> s2 >> m0 >> m1 >> m2 && (version == 2 || f >> kind)) {
+      if (p < 0 || p > 2 || N < 1 || N > SEM_MAX_N || !(best == 0 || best == 1 || best == 3) || s0 < least || s0 > 1 ||
+          !((s1 >= least && s1 <= 1) ||
+            (s1 == kTensorShape && ax_tensor_available(N, static_cast<sem_prec>(p), SEM_AX_OTF))) ||
+          s2 < least || s2 > 0 || kind < 0 || kind >= kTuneKinds)
         return fail(SEM_ERR_ARG, "corrupt tuning table");
-      TuneSlot& t = g_tune[p][N];
-      t.valid = true;
-      t.best = static_cast<sem_ax_variant>(best);
-      t.shape[0] = s0;
-      t.shape[1] = s1;
-      t.shape[2] = s2;
-      t.ms[0] = m0;
-      t.ms[1] = m1;
-      t.ms[2] = m2;
+      for (int q = 0; q < kTuneKinds; ++q) {
+        if (version != 2 && q != kind) continue;
+        TuneSlot& t = g_tune[p][q][N];
+        t.valid = true;
+        t.best = static_cast<sem_ax_variant>(best);
+        t.shape[0] = s0;
+        t.shape[1] = s1;
+        t.shape[2] = s2;
+        t.ms[0] = m0;
+        t.ms[1] = m1;
+        t.ms[2] = m2;
+      }
     }
     return SEM_OK;
   });

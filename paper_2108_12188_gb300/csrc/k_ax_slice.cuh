@@ -496,6 +496,7 @@ struct SliceShape {
   static constexpr int kW = slice_width(NP);   // an element takes kW of the block's 8 points per direction,
   static constexpr int kSub = 8 / kW;          // so a block holds kSub^3 elements at a time
   static constexpr int kElems = kSub * kSub * kSub;
+  static_assert(kElems == ax_slice_elements(NP - 1), "elements per block");
   static constexpr int kPlanes = kSub > 1 ? 8 : NP;      // k-planes of the block that hold points
   static constexpr int kWarps = (kPlanes + 1) / 2;       // a warp takes two (two j-planes in the k contractions)
   static constexpr int kThreads = 32 * kWarps;

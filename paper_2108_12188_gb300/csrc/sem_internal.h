@@ -145,6 +145,8 @@ inline int64_t factor_stride(int Np, bool fp32) {
 // N = 1 the FP64 differences of equal values are exact zeros, which fixed-point factors do not keep on
 // stretched elements (relative error 1.4e-15 against 1.2e-16 at aspect ratio 100).
 __host__ __device__ constexpr bool ax_slice_order(int N) { return N == 3 || (N >= 5 && N <= 7) || (N >= 9 && N <= 11); }
+// Elements a block of it takes.
+constexpr int ax_slice_elements(int N) { return N <= 3 ? 8 : 1; }
 // SEM_F64X with stored factors runs there too where that is the faster of the two, and the more accurate
 // (A_L at 16.8M points in ms, slices against double-float: N = 7 0.344 and 0.409, a CG iteration 0.578 and
 // 0.643; N = 11 0.92 and 1.20, 1.31 and 1.95; but N = 3 0.36 and 0.27, N = 5 0.79 and 0.38, N = 6 0.62 and
