@@ -224,7 +224,7 @@ sem_status launch_ax_any(sem_mesh m, sem_prec prec, sem_ax_variant v, bool cg, A
   const bool fp64_data = prec != SEM_F32;
   a.coef = fp64_data ? static_cast<const void*>(m->coef64) : static_cast<const void*>(m->coef32);
   a.G = stored_factors(m, prec, &a.g_pairs);
-  if (cg && a.g_pairs && f64x_on_slices(m->N)) {  // (the pairs are for the plain operator, f64x_plain_pairs)
+  if ((cg || a.as_cg) && a.g_pairs && f64x_on_slices(m->N)) {  // (the pairs are for the plain operator, f64x_plain_pairs)
     a.G = m->GI;
     a.g_pairs = false;
   }
@@ -904,10 +904,12 @@ sem_status cg_start(sem_cg c, const void* b, void* x, bool x0_is_zero, cudaStrea
     // iterations run in double-float arithmetic: a restart after the recursive residual has
     // converged then replaces it by the true residual b - A x, and the solve corrects the
     // double-float operator's own rounding (about 1e-14 of |A| |x|) instead of stalling on it. (Where
-    // f64x_on_slices both are the same operator.)
+    // f64x_on_slices the iterations run that operator.)
     sem_prec rp = c->prec;
     sem_ax_variant rv = c->variant;
-    if (rp == SEM_F64X && !(rv == SEM_AX_STORED && f64x_on_slices(m->N) && !m->Gx)) {
+    if (rp == SEM_F64X && rv == SEM_AX_STORED && f64x_on_slices(m->N)) {
+      a.as_cg = true;
+    } else if (rp == SEM_F64X) {
       rp = SEM_F64;
       if (rv == SEM_AX_STORED && !has_factors(m, SEM_F64)) rv = SEM_AX_OTF;
     }

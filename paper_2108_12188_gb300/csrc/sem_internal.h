@@ -318,6 +318,7 @@ struct AxLaunch {
   void* w;            // output
   const void* G;      // stored factors or null
   bool g_pairs;       // SEM_F64X: G holds float pairs (high, low) instead of the FP64 operator's factors
+  bool as_cg;         // SEM_F64X, plain mode: the factors of CG mode (f64x_on_slices: fixed point, not pairs)
   const int* gexp;    // exponents of fixed-point factors (ax_slice_order)
   const GeoElement* geo;  // elements for fixed-point factors rebuilt on the fly, or null
   const void* coef;   // trilinear coefficients (otf)
