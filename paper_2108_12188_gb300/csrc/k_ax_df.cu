@@ -9,14 +9,10 @@ namespace {
 template <int NP>
 struct DfStored {
   static sem_status run(int N, bool cg, const AxLaunch& a, cudaStream_t s) {
-    if constexpr (f64x_on_slices(NP - 1)) {
-      return launch_ax_slice(N, cg, a, s);
-    } else {
-      if (a.g_pairs)
-        return cg ? launch_df_t<NP, true, kGkPairs>(N, a, s) : launch_df_t<NP, false, kGkPairs>(N, a, s);
-      constexpr int kGk = ax_slice_order(NP - 1) ? kGkFixed : kGkF64;
-      return cg ? launch_df_t<NP, true, kGk>(N, a, s) : launch_df_t<NP, false, kGk>(N, a, s);
-    }
+    static_assert(!f64x_on_slices(NP - 1), "in k_ax_df_hi.cu");
+    if (a.g_pairs) return cg ? launch_df_t<NP, true, kGkPairs>(N, a, s) : launch_df_t<NP, false, kGkPairs>(N, a, s);
+    constexpr int kGk = ax_slice_order(NP - 1) ? kGkFixed : kGkF64;
+    return cg ? launch_df_t<NP, true, kGk>(N, a, s) : launch_df_t<NP, false, kGk>(N, a, s);
   }
 };
 

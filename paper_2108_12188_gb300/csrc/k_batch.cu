@@ -296,9 +296,9 @@ __global__ void __launch_bounds__(kBatchThreads) k_update_batch(const BatchTable
       d->up_part[2 * c] = v[0];
       d->up_part[2 * c + 1] = v[1];
       __threadfence();
-      const unsigned t = atomicAdd(&st->ticket[1], 1u);
+      const unsigned t = atomicAdd(&st->ticket[0], 1u);
       last = t == static_cast<unsigned>(d->up_cnt - 1);
-      if (last) st->ticket[1] = 0u;
+      if (last) st->ticket[0] = 0u;
     }
     __syncthreads();
     if (last) {
@@ -350,10 +350,10 @@ __global__ void __launch_bounds__(kBatchThreads) k_flush_batch(const BatchTable*
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
-      const unsigned t = atomicAdd(&st->ticket[4], 1u);
+      const unsigned t = atomicAdd(&st->ticket[3], 1u);
       last = t == static_cast<unsigned>(d->up_cnt - 1);
       if (last) {
-        st->ticket[4] = 0u;
+        st->ticket[3] = 0u;
         st->alpha = 0.0;
       }
     }

@@ -134,7 +134,7 @@ __global__ void k_cg_init(int64_t n, const T* __restrict__ b, const T* __restric
   }
   double v[3] = {rz.value(), rr.value(), bb.value()};
   block_sums<3, kThreads>(v, sRed);
-  if (publish_partials<3>(v, partials, &st->ticket[2])) {
+  if (publish_partials<3>(v, partials, &st->ticket[1])) {
     partial_sums<3, kThreads>(partials, gridDim.x, v, sRed);
     const double srz = v[0], srr = v[1], sbb = v[2];
     if (threadIdx.x == 0) {
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 5 : 4) k_cg_update(
     v[1] = rr.value();
   }
   block_sums<2, kThreads>(v, sRed);
-  if (publish_partials<2>(v, partials, &st->ticket[1])) {
+  if (publish_partials<2>(v, partials, &st->ticket[0])) {
     partial_sums<2, kThreads>(partials, gridDim.x, v, sRed);
     const double srz = v[0], srr = v[1];
     if (threadIdx.x == 0) {
@@ -428,10 +428,10 @@ __global__ void k_cg_flush(int64_t n, T* __restrict__ x, const T* __restrict__ p
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    const unsigned int t = atomicAdd(&st->ticket[4], 1u);
+    const unsigned int t = atomicAdd(&st->ticket[3], 1u);
     last = (t == gridDim.x - 1);
     if (last) {
-      st->ticket[4] = 0u;
+      st->ticket[3] = 0u;
       st->alpha = 0.0;
     }
   }
@@ -472,7 +472,7 @@ __global__ void k_ir_residual(int64_t n, const double* __restrict__ b, const dou
   }
   double v[2] = {rr, bb};
   block_sums<2, kThreads>(v, sRed);
-  if (publish_partials<2>(v, partials, &st->ticket[3])) {
+  if (publish_partials<2>(v, partials, &st->ticket[2])) {
     partial_sums<2, kThreads>(partials, gridDim.x, v, sRed);
     const double srr = v[0], sbb = v[1];
     if (threadIdx.x == 0) {
@@ -511,7 +511,7 @@ __global__ void k_cg_replace(int64_t n, const float* __restrict__ rnew, float* _
   }
   double v[2] = {rz.value(), rr.value()};
   block_sums<2, kThreads>(v, sRed);
-  if (publish_partials<2>(v, partials, &st->ticket[2])) {
+  if (publish_partials<2>(v, partials, &st->ticket[1])) {
     partial_sums<2, kThreads>(partials, gridDim.x, v, sRed);
     const double srz = v[0], srr = v[1];
     if (threadIdx.x == 0) {

@@ -123,7 +123,7 @@ void build_gs_host(const Topology& T, GsHost& out);
 struct CgScalars {
   double rho, alpha, beta, pw, rz, rr, bb, rtol2;
   int iter, max_iter, done, status;  // status: 0 running, SEM_OK converged, else sem_status
-  unsigned int ticket[5];            // last-block-done counters (reset by the last block)
+  unsigned int ticket[4];            // last-block-done counters (reset by the last block)
 };
 
 // Element stride (in elements of the factor type) of the mesh's stored-factor arrays: the six
