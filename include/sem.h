@@ -90,7 +90,8 @@ typedef enum { SEM_AX_STORED = 0, SEM_AX_OTF = 1, SEM_AX_AUTO = 2, SEM_AX_OTF_SC
 #define SEM_MESH_F64_STORED 1u /* G for SEM_F64: 48 bytes per local point (FP64; 64-bit fixed point at orders 3, 5-7, 9-11,
                                 * where a solver with use_graph = 2 adds the FP64 values if it runs in the persistent kernel) */
 #define SEM_MESH_F32_STORED 2u /* G in FP32: 24 bytes per local point */
-#define SEM_MESH_OTF_SCALE 4u  /* w_i w_j w_k / det J per point, FP64 and FP32: 12 bytes per local point */
+#define SEM_MESH_OTF_SCALE 4u  /* w_i w_j w_k / det J per point, FP64 and FP32: 12 bytes per local point (FP32 only, 4 bytes, where
+                                * SEM_F64 on the fly runs on the tensor cores and rebuilds it) */
 #define SEM_MESH_F64X_STORED 8u /* G as float pairs (high, low: 48 significant bits) for SEM_F64X: 48 bytes
                                  * per local point; without it SEM_F64X splits the FP64 factors itself (orders 7, 11: the array
                                  * of SEM_MESH_F64_STORED, held once; order 7 below 2560 elements

@@ -196,7 +196,7 @@ bool has_factors(sem_mesh m, sem_prec prec) {
   bool pairs;
   return stored_factors(m, prec, &pairs) != nullptr;
 }
-bool has_scales(sem_mesh m) { return m->scale64 != nullptr; }
+bool has_scales(sem_mesh m) { return m->scale32 != nullptr; }
 
 // Resolves SEM_AX_AUTO and picks the tuned block shape.
 void resolve_variant(sem_mesh m, sem_prec prec, sem_ax_variant v, sem_ax_variant* out_v, int* out_shape) {
@@ -233,7 +233,7 @@ sem_status launch_ax_any(sem_mesh m, sem_prec prec, sem_ax_variant v, bool cg, A
   a.scale = fp64_data ? static_cast<const void*>(m->scale64) : static_cast<const void*>(m->scale32);
   if (v == SEM_AX_STORED && !a.G)
     return fail(SEM_ERR_ARG, "stored factors of this precision were not requested at mesh creation");
-  if (v == SEM_AX_OTF_SCALE && !a.scale)
+  if (v == SEM_AX_OTF_SCALE && !has_scales(m))
     return fail(SEM_ERR_ARG, "per-point scales were not requested at mesh creation (SEM_MESH_OTF_SCALE)");
   if (prec == SEM_F64X) return launch_ax_f64x(m->N, v, cg, a, s);
   if (a.shape == kTensorShape && ax_tensor_available(m->N, prec, v)) return launch_ax_tc(m->N, cg, a, s);
@@ -480,6 +480,10 @@ extern "C" sem_status sem_mesh_create(int N, int64_t nv, const double* vert_xyz,
       dfree(m->geo, s);
       m->geo = nullptr;
       acc -= static_cast<size_t>(E) * sizeof(GeoElement);
+    }
+    if (m->geo && m->scale64) {  // FP64 on the fly rebuilds them
+      dfree(m->scale64, s);
+      acc -= static_cast<size_t>(E * P) * sizeof(double);
     }
     if (bad_h & 1) return cleanup(fail(SEM_ERR_MESH, "det J <= 0 (inverted or degenerate element)"));
   #undef SEM_STEP

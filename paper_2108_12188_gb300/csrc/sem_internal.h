@@ -269,7 +269,7 @@ struct sem_mesh_s {
   sem::GeoElement* geo = nullptr;  // [E] elements for factors rebuilt in fixed point (ax_slice_order), or null: not this mesh
   float* G32 = nullptr;       // [E][factor_stride] (the [6][P] block, padded to 16 bytes) or null
   float* Gx = nullptr;        // [E][6][P] float pairs (high, low) of G for SEM_F64X (f64x_on_slices: only f64x_plain_pairs), or null
-  double* scale64 = nullptr;  // [n] w_i w_j w_k / det J (SEM_MESH_OTF_SCALE) or null
+  double* scale64 = nullptr;  // [n] w_i w_j w_k / det J (SEM_MESH_OTF_SCALE) or null (also with geo: rebuilt, not read)
   float* scale32 = nullptr;
   int32_t* gs_rec[sem::kGsClasses] = {};  // gather-scatter plan (views in gs)
   uint8_t* gs_msk[sem::kGsClasses] = {};
