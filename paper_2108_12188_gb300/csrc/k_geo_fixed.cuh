@@ -71,12 +71,13 @@ struct __align__(16) GeoElement {
   int up;             // (c_a . c_b / 2^64) F / 2^(64 - up) uses 62 bits; 8 bits up: its right shift to X less the row scales
 };
 constexpr int kGeoNone = 1 << 20;
-// Bits of det J an element has to have in fixed point, and the most that `up` may be; beyond, the factors would
-// come out less exact than FP64 has them, and a mesh with such an element keeps k_ax. Relative rms error of the
-// factors against 80 bits, here and in FP64, over 200 elements with vertices moved by 15%, N = 9: 3.0e-17 and 2.1e-16
-// (55 bits, up 9), at an aspect ratio of 10 5.7e-17 and 2.1e-16 (52, 9), sheared by 5 1.2e-16 and 2.6e-16 (53, 9), at an
-// aspect ratio of 100 3.2e-16 and 2.4e-16 (49, 8); moved by 30% 1.7e-16 and 2.1e-16 (52, 12), N = 11 3.3e-16 and 2.1e-16 (51, 13).
-constexpr int kGeoBits = 52, kGeoUp = 14;
+// Bits of det J an element has to have in fixed point, and the most that `up` and the rows' shifts may be; beyond, the factors
+// would come out less exact than FP64 has them, and a mesh with such an element keeps k_ax. Relative rms error of the
+// factors against 80 bits, here and in FP64, over 200 elements with vertices moved by 15%, N = 9: 3.9e-17 and 2.5e-16 (up 9),
+// ten times as long along r, s or t 3.9e-17 or less and 2.5e-16, along t 30 times 7.5e-17 and 2.3e-16 (shift 14) and 100 times 1.4e-16 and
+// 2.2e-16 (shift 15; 300 times, 17, 3.7e-16), sheared by 5 4.7e-17 and 2.9e-16; moved by 30% 1.6e-16 and 2.4e-16 (up 12), N = 11 2.2e-16
+// and 2.4e-16 (up 12; with 14 3.2e-16).
+constexpr int kGeoBits = 52, kGeoUp = 12, kGeoShift = 15;
 
 // Node values: coordinates in units of 2^-62, weights times 2^c (c: fixed_row_scale) below 2^62.
 template <int NP>
@@ -119,7 +120,7 @@ SEM_HD int geo_scale(GeoElement& g, int coef, const int (&row)[3], int det, int 
   const int up = 62 - (all + unit);
   g.sg = 59 - top < unit + up - 2 ? 59 - top : unit + up - 2;
   g.up = up | (unit + up - g.sg) << 8;
-  bool ok = d >= kGeoBits && d <= 61 && g.s >= 0 && g.s <= 29 && g.s2 <= 29 && up >= 0 && up <= kGeoUp &&
+  bool ok = d >= kGeoBits && d <= 61 && g.s >= 0 && g.s <= kGeoShift && g.s2 <= kGeoShift && up >= 0 && up <= kGeoUp &&
             unit + up - g.sg <= 40;
   for (int v : {coef, row[0], row[1], row[2], det, top, all}) ok = ok && v > -200 && v < 200;
   if (!ok) g.sg = kGeoNone;
@@ -151,6 +152,8 @@ SEM_HD GeoEntry geo_entry(const GeoElement& e, int d, int c, const Fx& v, int on
     FxSum t;
     t.add(ay, bz);
     t.sub(az, by);
+    // (of two short vectors the difference is small and sh large: the low by low products count)
+    t.m += (static_cast<long long>(ay.l) * bz.l - static_cast<long long>(az.l) * by.l) >> 32;
     return t.get_shl(sh);
   };
   if (d == 0) *xt = {at(m0, m1, c), fx_split(fx_shl(at(k0, 6, c), 2))};
