@@ -1,5 +1,5 @@
-// Local operator A_L = D^T G D (Eq. 4, Section 3.1) for FP64 data, with stored factors (but at N = 7,
-// where k_ax_slice takes them, see f64x_on_slices) or
+// Local operator A_L = D^T G D (Eq. 4, Section 3.1) for FP64 data, with stored factors (but at N = 7
+// and 11, where k_ax_slice takes them, see f64x_on_slices) or
 // factors rebuilt on the fly (Section 5.1), computed in double-float arithmetic on the FP32
 // pipes (k_df.cuh): GB300 issues FP32 FMAs 64 times faster than FP64 ones, and the FP64
 // kernel is bound by the FP64 pipe. The kernel template is shared by four translation units

@@ -27,19 +27,21 @@
 // 2^58, so its digits are cut without another scaling. The three transposed contractions are added
 // as integers and rounded to FP64 once.
 //
-// What bounds it: GB300's integer instructions, 64 a clock per SM whatever their kind, with the
-// mma.sync and FP32 ones beside them (about 360 instructions per point, 46% of the issue slots, 0.46 of
-// the HBM time). 16.8M points, N = 7: 1.502 ms in FP64 (k_ax, 95% of the FP64 peak by Eq. 11 flops) ->
-// 0.344 ms. In CG mode with the fused prologue 0.414 ms; it takes 0.02 ms from the operator's earlier
-// unfused form (0.394) and saves 0.067 in the update kernel: one Jacobi-CG iteration 1.793 -> 0.578 ms.
+// What bounds it: dependent integer work. Of 371 instructions per point (429 in CG mode) 154 (168) run on the ALU, 134 (150) are
+// integer and FP32 multiply-adds of the heavy FMA pipe, 25.5 mma.sync. A probe of either kind or both mixed ran 64 lanes a
+// clock per SM; at that rate the two take 72% of the time (66%), with 38% and 45% of their pipes' cycles, and what is left is
+// latency: four warps per scheduler (128 registers) that wait on the instruction before (1.8 of 7 stalled), on the pipes
+// (1.1), on barriers and shared memory. 16.8M points, N = 7: 1.497 ms in FP64 (k_ax, 95% of the FP64 peak by Eq. 11 flops) ->
+// 0.337 ms, 0.46 of the HBM bandwidth. In CG mode with the fused prologue 0.411 ms (0.62); the prologue takes 0.02 ms and saves
+// 0.067 in the update kernel: one Jacobi-CG iteration 1.779 -> 0.554 ms.
 //
 // On the fly (Section 5.1's rematerialised factors) the same kernel fills its factor buffer from the element's
 // coefficients, with about 700 instructions per point on the same pipes, still far below the 45 FP64 instructions
-// of k_ax for it. A_L in ms, k_ax and this kernel, 16M points: N = 3 2.72 and 1.10, N = 5 3.07 and 1.60, N = 6 2.98 and
-// 1.37, N = 7 2.63 and 0.90, N = 9 3.62 and 2.08, N = 10 3.13 and 1.78, N = 11 3.49 and 1.46 (of these the factors take
+// of k_ax for it. A_L in ms, k_ax and this kernel, 16.0 to 17.6M points: N = 3 2.84 and 1.17, N = 5 3.31 and 1.74, N = 6 3.23 and
+// 1.49, N = 7 2.89 and 0.99, N = 9 4.07 and 2.36, N = 10 3.13 and 1.76, N = 11 3.49 and 1.45 (of these the factors take
 // 0.5 ms, the row tables 0.05 and at N = 3 0.2); with the per-point scale of SEM_AX_OTF_SCALE, which is not read
-// here, 2.31, 2.67, 2.58, 2.30, 3.18, 2.75 and 3.15 before. Error against FP64 torch as with k_ax (N = 9 1.2e-15 and
-// 1.3e-15, N = 7 9.0e-16 and 9.3e-16).
+// here, k_ax takes 0.8 to 0.9 of that. Error against long double (jittered elements, random u, N = 9) as with k_ax or below:
+// 1.9e-16 and 2.6e-16, stored 2.4e-16 and 2.6e-16.
 //
 // Error against 64 bits (relative 2-norm of w, N = 7, jittered elements, CPU model of both
 // kernels against an 80-bit reference; k_ax in brackets): random u 8e-17 (1.8e-16), a sine over 8^3
@@ -534,7 +536,7 @@ __device__ __forceinline__ unsigned over_element(unsigned v, F&& op) {
 // Warp q holds the points of planes k = 2q and 2q + 1, lane (j = lane / 4, i = 2 (lane % 4) + {0, 1}), both
 // of one element; lanes and planes beyond an element's points hold zeros. Phases of a group:
 //   0  u (CG, fused_cg: the previous iteration's x += alpha p, p = M^-1 r + beta p) to registers; largest
-//      exponent; digits of U to shared memory
+//      exponent and how many threads come near it (kNear); digits of U to shared memory
 //   1  k-lines (a warp takes j = 2q, 2q + 1): ut, exchanged through shared memory; i-rows and j-lines
 //      of the own planes: ur, us stay in the lane that owns the point; largest magnitude
 //   2  geometry; digits of vt to shared memory
@@ -542,8 +544,7 @@ __device__ __forceinline__ unsigned over_element(unsigned v, F&& op) {
 //      barrier) on k-lines, exchanged back; w
 // The factors of the next group arrive by one TMA bulk copy during phase 3 and the next phase 0.
 // OTF: the factors are rebuilt (OtfGeometry: row tables in phase 0, the factors before phase 1) instead of
-// copied; three blocks per SM there (168 registers; N = 7 0.91 ms with four, 0.90 with three, N = 3 100 and 96 us at
-// 1.3M points), four at N = 5, whose blocks of 96 threads have the registers (CG 2.19 ms with three, 2.13 with four).
+// copied; three blocks per SM there (168 registers; N = 7 1% slower with four, N = 3 100 and 96 us at 1.3M points), four at N = 5, whose blocks of 96 threads have the registers (CG 2.19 ms with three, 2.13 with four).
 template <int NP, bool CG, bool OTF>
 __global__ void __launch_bounds__(SliceShape<NP>::kThreads, OTF && NP != 6 ? 3 : 4)
     k_ax_slice(const __grid_constant__ GllParam<NP, double> tab, const __grid_constant__ SliceTab<NP> sl,

@@ -4,8 +4,8 @@
 // g + 1 of them; the groups from magic_groups on exceed the 2^22 that fit on top of kMagic and are split
 // in FP32.
 //
-// 16.8M points, FP64 (k_ax) against this kernel: N = 9 2.03 and 1.51 ms, N = 10 1.79 and 1.08, N = 11 2.06 and
-// 0.84; 216 elements at N = 11 72 and 35 us. It is bound as k_ax_slice is, and works on 256 points of
+// 17.6, 16.2 and 16.0M points, FP64 (k_ax) against this kernel: N = 9 2.03 and 1.47 ms, N = 10 1.79 and 1.03, N = 11 2.06 and
+// 0.81; 180 elements at N = 11 68 and 30 us. It is bound as k_ax_slice is, and works on 256 points of
 // every plane where the element has (N + 1)^2 (N = 9 100), with 9 to 12 warps per SM.
 #pragma once
 

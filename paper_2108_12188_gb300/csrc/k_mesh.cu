@@ -325,8 +325,8 @@ __device__ __forceinline__ void sincos_small(const TaylorTab& k, int terms, doub
 // are 190 of them. Along a row x is linear in xi, so sin(a pi x) is a rotation of the row's midpoint value
 // by angles +-a pi B xi_i, whose sines and cosines are short sums and serve two points each (the GLL nodes
 // are symmetric); the midpoints follow the same way from one value per k-plane. Along the row det J is a
-// quadratic in xi, formed once. 48 instructions per point at N = 9: with the gather-scatter 2.14 ->
-// 0.85 ms at 8.0M points (0.72 of it at the FP64 rate a chain of multiply-adds reaches). Elements too large for the short sums (|a B| > 1/4) take sincospi and sinpi.
+// quadratic in xi, formed once. 55 of them per point at N = 9: with the gather-scatter 2.14 ->
+// 0.83 ms at 8.0M points, the FP64 pipe 90% busy. Elements too large for the short sums (|a B| > 1/4) take sincospi and sinpi.
 __global__ void k_rhs_local(const __grid_constant__ GllAll tab, const __grid_constant__ TaylorTab tay, int Np, int epb,
                             int split, int chunk, int64_t E, const double* __restrict__ coef, int fa, int fb, int fc,
                             double* __restrict__ out) {

@@ -138,19 +138,20 @@ inline int64_t factor_stride(int Np, bool fp32) {
 // the fly on meshes whose elements fixed point rebuilds as exactly as FP64 (sem_mesh_s::geo).
 // Their meshes keep G as 64-bit fixed point instead of FP64, in the same bytes: X = G_ab 2^(sg + c_a + c_b),
 // |X| <= 2^59, as 32-bit signed halves (low, high), with sg per element and c = fixed_row_scale of the
-// point's index along each direction. Stored, at 16.8M points the FP64 kernel against this one: N = 3 1.12 and
-// 0.36 ms, N = 5 1.50 and 0.75, N = 6 1.52 and 0.59, N = 7 1.50 and 0.34, N = 9 2.03 and 1.51, N = 10 1.79 and
-// 1.08, N = 11 2.06 and 0.85; on the fly 1.7 to 2.9 times (k_ax_slice.cuh). N = 2, 4 and 8 fill too little of the boxes of 8 or 16 points a side that the
-// tensor cores work on (N = 2 0.86 against 0.93 ms, N = 4 1.13 against 1.31; 729 of 2304 points at N = 8). At
+// point's index along each direction. Stored, at 16.0 to 17.6M points the FP64 kernel against this one: N = 3 1.11 and
+// 0.36 ms, N = 5 1.50 and 0.80, N = 6 1.52 and 0.62, N = 7 1.50 and 0.34, N = 9 2.03 and 1.47, N = 10 1.79 and
+// 1.03, N = 11 2.06 and 0.81; on the fly 1.7 to 2.9 times (k_ax_slice.cuh). N = 2 and 4 fill too little of the boxes of 8
+// points a side that the tensor cores work on (N = 2 0.86 against 0.93 ms, N = 4 1.13 against 1.31); N = 8, 729 of 2304 points, was not
+// measured. Small meshes gain too (1 to 2197 elements, every order, both factors: 0.4 to 0.93 of the FP64 kernel's time). At
 // N = 1 the FP64 differences of equal values are exact zeros, which fixed-point factors do not keep on
 // stretched elements (relative error 1.4e-15 against 1.2e-16 at aspect ratio 100).
 __host__ __device__ constexpr bool ax_slice_order(int N) { return N == 3 || (N >= 5 && N <= 7) || (N >= 9 && N <= 11); }
 // Elements a block of it takes.
 constexpr int ax_slice_elements(int N) { return N <= 3 ? 8 : 1; }
 // SEM_F64X with stored factors runs there too where that is the faster of the two, and the more accurate
-// (A_L at 16.8M points in ms, slices against double-float: N = 7 0.344 and 0.409, a CG iteration 0.578 and
-// 0.643; N = 11 0.92 and 1.20, 1.31 and 1.95; but N = 3 0.36 and 0.27, N = 5 0.79 and 0.38, N = 6 0.62 and
-// 0.50, N = 9 1.45 and 0.73, N = 10 1.13 and 0.71).
+// (A_L at 16.0 to 17.6M points in ms, slices against double-float: N = 7 0.337 and 0.406, a CG iteration 0.554 and
+// 0.623; N = 11 0.81 and 1.14, 1.18 and 1.91; but N = 3 0.36 and 0.26, N = 5 0.80 and 0.37, N = 6 0.62 and
+// 0.49, N = 9 1.47 and 0.78, N = 10 1.03 and 0.67).
 __host__ __device__ constexpr bool f64x_on_slices(int N) { return N == 7 || N == 11; }
 // The plain operator (sem_ax) keeps double-float factors for meshes of fewer elements than this at N = 7: its blocks
 // take two elements and fill one or two waves where the slices take two or three. Slices and double-float in us:
@@ -264,7 +265,7 @@ struct sem_mesh_s {
   double* coef64 = nullptr;   // [E][24] trilinear coefficients a0..a7 (x, y, z)
   float* coef32 = nullptr;    // [E][24] rounded to FP32
   double* G64 = nullptr;      // [E][6][P] or null (ax_slice_order: once a solver has taken use_graph = 2)
-  int2* GI = nullptr;         // [E][6][P] fixed-point factors (ax_slice_order; at N = 7 for SEM_F64X too) or null
+  int2* GI = nullptr;         // [E][6][P] fixed-point factors (ax_slice_order; f64x_on_slices: for SEM_F64X too) or null
   int* gexp = nullptr;        // [E] their exponents sg
   sem::GeoElement* geo = nullptr;  // [E] elements for factors rebuilt in fixed point (ax_slice_order), or null: not this mesh
   float* G32 = nullptr;       // [E][factor_stride] (the [6][P] block, padded to 16 bytes) or null
